@@ -225,7 +225,7 @@ cfi_dense_split_kernel(DevLayer L, const __grid_constant__ CUtensorMap map_w, co
             tma_load_2d(dst + kSpWBytes, &map_x, full0 + 8 * s, (kb0 + i) * kSpK, b0);
             issued = i + 1;  // (the first ring round has no wait that could fail, so no stage is left with only its weight box)
         }
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1 && elect_one()) {
         // ---------------------------------------------------------------- first MMA issuer: Wd x [x; x_lo], N = 2 BT.
         // (The two issuers are written out separately: a thread gets a tcgen05 instruction accepted only about every
         // 150 cycles, and any branch in this loop costs more.  A stage's "ready" barrier completes only after its
@@ -245,7 +245,7 @@ cfi_dense_split_kernel(DevLayer L, const __grid_constant__ CUtensorMap map_w, co
             umma_commit(empty0 + 8 * s);
         }
         umma_commit(accum);  // also after a failed wait: the arrival then tells when the MMAs issued so far are done
-    } else if (warp == 2 && lane == 0) {
+    } else if (warp == 2 && elect_one()) {
         // ---------------------------------------------------------------- second MMA issuer: w_lo x x, N = BT
         constexpr uint32_t idesc = sp_instr_desc(BT);
         const uint32_t acc = tmem_base + (uint32_t)(2 * BT);

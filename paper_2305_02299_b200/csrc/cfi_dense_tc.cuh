@@ -109,6 +109,14 @@ __device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t desc_a, uint
         "l"(desc_a), "l"(desc_b), "r"(kTcInstrDesc), "r"(accumulate), "r"(0u)
         : "memory");
 }
+// True in one lane of a converged warp.  The tensor-core instructions take their descriptors and barrier addresses from
+// uniform registers; behind this predicate the compiler knows that a single lane runs the branch, where behind
+// `lane == 0` it has to allow for several and guards every such instruction with a loop over the lanes.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(p));
+    return p != 0;
+}
 __device__ __forceinline__ void umma_commit(uint32_t mbar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar) : "memory");
 }
@@ -308,7 +316,7 @@ cfi_dense_tc_kernel(DevLayer L, const __grid_constant__ CUtensorMap map_x, const
             if (kb >= kTcStages) tma_load_2d(b_dst, &map_w, full0 + 8 * s, (kb0 + kb) * kTcK, n0);
             issued = kb + 1;  // (the first ring round has no wait that could fail, so no stage is left with only its weight box)
         }
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1 && elect_one()) {
         // ---------------------------------------------------------------- MMA issuer
         for (int kb = 0; kb < k_blocks && ok; ++kb) {
             const int s = kb % kTcStages;

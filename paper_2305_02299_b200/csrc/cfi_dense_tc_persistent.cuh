@@ -108,7 +108,7 @@ cfi_dense_tc_persistent_kernel(DevLayer L, const __grid_constant__ CUtensorMap m
                 issued = g + 1;
             }
         }
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1 && elect_one()) {
         // ---------------------------------------------------------------- MMA issuer
         uint32_t g = 0, i = 0;  // K blocks and tiles so far
         for (int t = first; t < n_tiles && ok; t += stride, ++i) {
