@@ -5,12 +5,18 @@
 // K largest gradient magnitudes among the inactive positions of live neurons -- and one selection per neuron (regrow
 // to the new fan-in k', or trim down to it).  All of them are "the m smallest of a set of (32-bit key, position)
 // pairs, ties to the smaller position", with key = the bits of |w| (a non-negative float orders like its bits) or
-// the complement of the bits of |grad| (so that a larger gradient is a smaller key).  They are done by radix
-// selection: four passes of 256-bin histograms over the digits of the key from the top, each pass narrowing to the
-// bin that holds the m-th element, then the ties on the final key are cut in position order.  For the two layer-wide
-// selections the last pass also lists the few elements that match the first three digits; when a list holds them all
-// (the rule), the position of the last tie taken is selected from it and the marking pass is elementwise; inputs with
-// very many equal keys overflow the list and are ranked with per-chunk tie counts and a prefix sum instead.
+// the complement of the bits of |grad| (so that a larger gradient is a smaller key).  Key and position together are one
+// 62-bit number, the composite, and no two elements share one, so ties need no ranking of their own.
+//
+// The two layer-wide selections are radix selections that stop sweeping the layer early.  One sweep counts the first 12
+// bits of the keys, which leaves about 1 % of the elements open; a second one lists those, and the rest is decided on
+// the lists.  Per neuron one 11-bit digit leaves a few dozen open, which are ranked against one another.  A layer with
+// so many equal keys that the open elements do not fit the lists takes further digits first, at last of the position.
+//
+// 4096 x 4096 at 80 %, K = 30 % of the weights, four kernels: 34 + 41 + 16 + 73 us, 0.20 ms with the host's wait
+// (before: four sweeps of 8-bit digits, flags for every entry and a four-digit selection per neuron, 12 kernels: 0.39 ms);
+// 3072 x 768 at 90 %: 17 + 19 + 13 + 19 us, 0.10 ms (0.17 ms).  Moved per entry: 9 bytes in each of the two sweeps and the
+// per-neuron step, and what changes: 30 against 50.
 //
 // Readings where Sec. 3.1 leaves a choice (the same as the CPU oracle used by the tests takes): already ablated
 // neurons stay out; a weight is salient if it is active and not among the K smallest, or inactive and among the K
@@ -22,538 +28,590 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
+#include <type_traits>
 
 namespace {
 
-constexpr int kThreads = 256, kChunk = 16 * kThreads;  // a block marks ties over 4096 consecutive positions
+constexpr int kThreads = 256;
+constexpr int kDigit = 12, kBins = 1 << kDigit;  // layer-wide digits
+constexpr int kKeyBits = 31, kPosBits = 31, kAllBits = kKeyBits + kPosBits;
 
-struct SelectState {
-    unsigned long long want;     // elements still to take inside the current prefix bin (1-based rank of the cut)
-    unsigned long long below;    // elements with a key below the current prefix
-    unsigned int prefix, prefix_mask;
-    unsigned int hist[256];
-    unsigned int blocks_done;    // blocks of the running histogram sweep that have added their counts (first state only)
-    // The last sweep also lists the elements that match the first three digits (key, position): a few hundred as a rule.
-    // If the list holds them all, the position of the last tie taken follows from it and the marking needs no ranking.
-    unsigned int listed;         // elements offered to the list (may exceed its capacity)
-    unsigned int last_tie;       // ties on the cut key are taken up to and including this position
-    unsigned int listed_all;     // 1: last_tie is valid
+// One layer-wide selection: the `want` smallest of its elements, as far as it is narrowed down.
+struct Select {
+    unsigned long long prefix;   // elements with (composite >> shift) < prefix are taken, > prefix are not, == are open
+    unsigned long long want;     // how many of the open ones are still to take
+    unsigned long long cut;      // after resolve_kernel: composite <= cut is taken
+    unsigned int count;          // open elements
+    unsigned int listed, listed_ties;  // entries of the two lists
+    int shift;
+    int on;                      // 0: nothing to select (K = 0 after clipping)
 };
 
-// Capacity of a selection's list: enough for ordinary key distributions, small against the layer; inputs with very many
-// equal keys overflow it and take the ranking path.
-__host__ __device__ inline unsigned int list_capacity(long long n) {
-    const long long c = n / 64;
-    return (unsigned int)(c < 64 ? 64 : c > 32768 ? 32768 : c);
-}
-
-struct Scalars {
-    long long active_total, inactive_total;
-    int k, k_new, live_before, live_after;
+struct StateHead {               // what the host reads back
+    Select sel[2];
+    unsigned long long active_total;
+    int live, k, blocks_done;
+    int listable;                // both selections' open elements fit their lists
+    int done;                    // resolve_kernel has run
+    int k_new, live_after;
+};
+struct State : StateHead {       // zeroed before the first sweep
+    alignas(16) unsigned int hist[2][kBins];
 };
 
-__device__ __forceinline__ unsigned int mag_bits(float v) { return __float_as_uint(fabsf(v)); }
-
-// h[bin] += 1 for every lane that takes part; lanes of the warp with the same bin are counted by one of them.  (The top
-// digits of float magnitudes fall into a handful of bins, and a plain atomic per lane would serialise on them.)
-__device__ __forceinline__ void hist_add(unsigned int* h, bool take, unsigned int bin) {
-    const unsigned int active = __ballot_sync(0xffffffffu, take);
-    if (take) {
-        const unsigned int peers = __match_any_sync(active, bin);
-        if ((int)(__ffs(peers) - 1) == (int)(threadIdx.x & 31)) atomicAdd(&h[bin], (unsigned int)__popc(peers));
-    }
+// 31-bit keys: the bits of |v| for a weight; for a gradient their complement, so that a larger one is a smaller key.
+__device__ __forceinline__ unsigned int weight_key(float v) { return __float_as_uint(v) & 0x7FFFFFFFu; }
+__device__ __forceinline__ unsigned int grad_key(float v) { return ~__float_as_uint(v) & 0x7FFFFFFFu; }
+__device__ __forceinline__ unsigned long long composite(unsigned int key, unsigned int pos) {
+    return ((unsigned long long)key << kPosBits) | pos;
+}
+// composite >> shift, with 32-bit arithmetic while the shift leaves key bits only.
+__device__ __forceinline__ unsigned long long composite_top(unsigned int key, unsigned int pos, int shift) {
+    if (shift >= kPosBits) return key >> (shift - kPosBits);
+    return composite(key, pos) >> shift;
 }
 
-__global__ void row_count_kernel(const uint8_t* mask, int out_f, int in_f, int* row_count) {
-    __shared__ int s;
-    const int r = blockIdx.x;
-    if (threadIdx.x == 0) s = 0;
-    __syncthreads();
-    int c = 0;
-    if ((in_f & 15) == 0) {  // 16 mask bytes per load; __vcmpne4 turns every nonzero byte into 0xff
-        const uint4* m16 = reinterpret_cast<const uint4*>(mask + (size_t)r * in_f);
-        for (int v = threadIdx.x; v < (in_f >> 4); v += blockDim.x) {
-            const uint4 m = m16[v];
-            c += (__popc(__vcmpne4(m.x, 0u)) + __popc(__vcmpne4(m.y, 0u)) + __popc(__vcmpne4(m.z, 0u)) + __popc(__vcmpne4(m.w, 0u))) >> 3;
+// VEC consecutive columns of a row: mask bytes (one per byte of m), weights, gradients.
+template <int VEC> struct Cols;
+template <> struct Cols<4> {
+    unsigned int m;
+    float4 w4, g4;
+    __device__ __forceinline__ void load_mask(const uint8_t* mask, size_t at, bool in) { m = in ? *reinterpret_cast<const unsigned int*>(mask + at) : 0u; }
+    __device__ __forceinline__ void load_values(const float* w, const float* grad, size_t at, bool in) {
+        w4 = g4 = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (in) {
+            w4 = *reinterpret_cast<const float4*>(w + at);
+            g4 = *reinterpret_cast<const float4*>(grad + at);
         }
-    } else {
-        for (int j = threadIdx.x; j < in_f; j += blockDim.x) c += mask[(size_t)r * in_f + j] ? 1 : 0;
     }
-    for (int off = 16; off > 0; off >>= 1) c += __shfl_down_sync(0xffffffffu, c, off);
-    if ((threadIdx.x & 31) == 0 && c) atomicAdd(&s, c);
+    __device__ __forceinline__ bool on(int e) const { return (m >> (8 * e)) & 0xFFu; }
+    __device__ __forceinline__ int count() const { return __popc(__vcmpne4(m, 0u)) >> 3; }
+    __device__ __forceinline__ float w(int e) const { return e == 0 ? w4.x : e == 1 ? w4.y : e == 2 ? w4.z : w4.w; }
+    __device__ __forceinline__ float g(int e) const { return e == 0 ? g4.x : e == 1 ? g4.y : e == 2 ? g4.z : g4.w; }
+};
+template <> struct Cols<1> {
+    unsigned int m;
+    float w1, g1;
+    __device__ __forceinline__ void load_mask(const uint8_t* mask, size_t at, bool in) { m = in ? mask[at] : 0u; }
+    __device__ __forceinline__ void load_values(const float* w, const float* grad, size_t at, bool in) {
+        w1 = in ? w[at] : 0.f;
+        g1 = in ? grad[at] : 0.f;
+    }
+    __device__ __forceinline__ bool on(int) const { return m != 0u; }
+    __device__ __forceinline__ int count() const { return m != 0u; }
+    __device__ __forceinline__ float w(int) const { return w1; }
+    __device__ __forceinline__ float g(int) const { return g1; }
+};
+
+// Sum over the block of one int per thread; slot alternates between calls so that one barrier per call is enough.
+template <int T>
+__device__ __forceinline__ int block_sum(int v, int (&part)[2][T / 32], int slot) {
+    v = __reduce_add_sync(0xffffffffu, v);
+    if ((threadIdx.x & 31) == 0) part[slot][threadIdx.x >> 5] = v;
     __syncthreads();
-    if (threadIdx.x == 0) row_count[r] = s;
+    int total = 0;
+#pragma unroll
+    for (int i = 0; i < T / 32; ++i) total += part[slot][i];
+    return total;
 }
 
-// Single block: totals, k, and the initial state of the two layer-wide selections (K clipped to both pools).
-__global__ void setup_kernel(const int* row_count, int out_f, int in_f, long long K, Scalars* sc, SelectState* st) {
-    __shared__ long long act;
-    __shared__ int live, k;
-    if (threadIdx.x == 0) act = 0, live = 0, k = 0;
-    __syncthreads();
-    long long my_act = 0;
-    int my_live = 0, my_k = 0;
-    for (int r0 = threadIdx.x; r0 < out_f; r0 += 8 * blockDim.x) {  // eight rows' loads in flight
-        int rc[8];
+// The bin of a histogram that holds the `want`-th element (1-based; the caller guarantees that there are so many), how
+// many elements the bins before it hold and how many it holds itself.  The whole block, T threads, the kPer consecutive bins v of each.
+struct Pick { unsigned int bin, below, count; };
+template <int T, int kPer>
+__device__ Pick block_pick(unsigned long long want, const unsigned int (&v)[kPer], unsigned int* part, Pick& out) {
+    const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+    unsigned int mine = 0;
 #pragma unroll
-        for (int u = 0; u < 8; ++u) rc[u] = r0 + u * blockDim.x < out_f ? row_count[r0 + u * blockDim.x] : 0;
-#pragma unroll
-        for (int u = 0; u < 8; ++u)
-            if (rc[u] > 0) my_act += rc[u], ++my_live, my_k = max(my_k, rc[u]);
-    }
-    for (int off = 16; off > 0; off >>= 1) {  // one set of atomics per warp
-        my_act += __shfl_down_sync(0xffffffffu, my_act, off);
-        my_live += __shfl_down_sync(0xffffffffu, my_live, off);
-        my_k = max(my_k, __shfl_down_sync(0xffffffffu, my_k, off));
-    }
-    if ((threadIdx.x & 31) == 0 && my_live) {
-        atomicAdd((unsigned long long*)&act, (unsigned long long)my_act);
-        atomicAdd(&live, my_live);
-        atomicMax(&k, my_k);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        sc->active_total = act;
-        sc->inactive_total = (long long)live * in_f - act;
-        sc->k = k, sc->live_before = live, sc->k_new = 0, sc->live_after = 0;
-        long long kk = K < 0 ? 0 : K;
-        if (kk > act) kk = act;
-        if (kk > sc->inactive_total) kk = sc->inactive_total;
-        for (int s = 0; s < 2; ++s)
-            st[s].want = (unsigned long long)kk, st[s].below = 0, st[s].prefix = 0, st[s].prefix_mask = 0, st[s].blocks_done = 0,
-            st[s].listed = 0, st[s].last_tie = 0, st[s].listed_all = 0;
-    }
-    for (int s = 0; s < 2; ++s)
-        for (int b = threadIdx.x; b < 256; b += blockDim.x) st[s].hist[b] = 0;
-}
-
-// One warp per selection: the bin that holds the `want`-th element (the first bin whose running count reaches it;
-// the last bin if none before it does); narrow the prefix to it and clear the histogram for the next pass.  Called by
-// the last block of a histogram sweep, after every block's counts have arrived.
-__device__ void pick_bin(int pass, SelectState* st) {
-    const int lane = threadIdx.x & 31;
-    const unsigned long long want = st->want;
-    unsigned int v[8];
-    unsigned long long mine = 0;
-#pragma unroll
-    for (int e = 0; e < 8; ++e) v[e] = __ldcg(&st->hist[8 * lane + e]), mine += v[e];
-    unsigned long long incl = mine;
+    for (int e = 0; e < kPer; ++e) mine += v[e];
+    unsigned int incl = mine;
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
-        const unsigned long long up = __shfl_up_sync(0xffffffffu, incl, off);
+        const unsigned int up = __shfl_up_sync(0xffffffffu, incl, off);
         if (lane >= off) incl += up;
     }
-    unsigned long long seen = incl - mine;  // count in the bins before this lane's
-    int found = 256;
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-        if (found == 256) {
-            if (seen + v[e] >= want) found = 8 * lane + e;
-            else seen += v[e];
-        }
-    }
-    int bin = found;
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) bin = min(bin, __shfl_xor_sync(0xffffffffu, bin, off));
-    if (bin > 255) bin = 255;
-    // `seen` of the lane that owns the bin is the count below it (for the last bin without a hit: lane 31 stopped there)
-    if (found == 256 && lane == 31) seen -= v[7];
-    const unsigned long long below_bin = __shfl_sync(0xffffffffu, seen, bin >> 3);
-#pragma unroll
-    for (int e = 0; e < 8; ++e) st->hist[8 * lane + e] = 0;
-    if (lane == 0 && want != 0) {
-        const int shift = 24 - 8 * pass;
-        st->want = want - below_bin;
-        st->below += below_bin;
-        st->prefix |= (unsigned int)bin << shift;
-        st->prefix_mask |= 255u << shift;
-    }
-}
-
-// The whole block (kThreads threads), one selection, after its last digit has been picked: if the list holds every
-// element that matched the first three digits, the ties on the cut key are all in it, and the position of the last tie
-// taken (the `want`-th in position order) is found by radix selection over the listed positions.  Then "taken" is
-// key < cut, or key == cut and position <= last_tie: the marking needs neither tie counts nor ranks.
-__device__ void find_last_tie(SelectState* st, const uint2* list, unsigned int cap) {
-    __shared__ unsigned int hist[256], warp_tot[kThreads / 32], res[2], ties_total;
-    const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
-    const unsigned int n = __ldcg(&st->listed);
-    if (n > cap) {  // the list overflowed (the same for the whole block): the ranking path decides
-        if (t == 0) st->listed_all = 0;
-        return;
-    }
-    const unsigned int cut = __ldcg(&st->prefix);
-    unsigned int want = (unsigned int)__ldcg(&st->want);  // ties to take
-    if (t == 0) ties_total = 0;
+    if (lane == 31) part[wid] = incl;
     __syncthreads();
-    unsigned int mine = 0;
-    for (unsigned int i = t; i < n; i += kThreads) mine += __ldcg(&list[i]).x == cut ? 1u : 0u;
+    unsigned int seen = incl - mine;
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) mine += __shfl_down_sync(0xffffffffu, mine, off);
-    if (lane == 0 && mine) atomicAdd(&ties_total, mine);
-    __syncthreads();
-    if (want == 0 || ties_total <= want) {  // selection off, or every tie is taken
-        if (t == 0) st->last_tie = 0xFFFFFFFFu, st->listed_all = 1;
-        return;
-    }
-    unsigned int prefix = 0, pmask = 0;
-    for (int pass = 0; pass < 4; ++pass) {
-        hist[t] = 0;
-        __syncthreads();
-        const int shift = 24 - 8 * pass;
-        for (unsigned int i = t; i < n; i += kThreads) {
-            const uint2 e = __ldcg(&list[i]);
-            if (e.x == cut && (e.y & pmask) == prefix) atomicAdd(&hist[(e.y >> shift) & 255u], 1u);
-        }
-        __syncthreads();
-        const unsigned int h = hist[t];
-        unsigned int incl = h;
+    for (int i = 0; i < T / 32; ++i) seen += i < wid ? part[i] : 0u;
+    if (seen < want && want <= (unsigned long long)seen + mine) {  // exactly one thread
+        bool found = false;
 #pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const unsigned int up = __shfl_up_sync(0xffffffffu, incl, off);
-            if (lane >= off) incl += up;
-        }
-        if (lane == 31) warp_tot[wid] = incl;
-        __syncthreads();
-        unsigned int before = 0;
-#pragma unroll
-        for (int i = 0; i < kThreads / 32; ++i) before += i < wid ? warp_tot[i] : 0u;
-        const unsigned int excl = before + incl - h;
-        if (excl < want && want <= excl + h) res[0] = (unsigned int)t, res[1] = excl;  // exactly one thread: want <= ties
-        __syncthreads();
-        prefix |= res[0] << shift;
-        pmask |= 255u << shift;
-        want -= res[1];
-        __syncthreads();  // res[] and hist[] are rewritten by the next pass
-    }
-    if (t == 0) st->last_tie = prefix, st->listed_all = 1;
-}
-
-// Histograms of digit `pass` (0 = top byte) for both layer-wide selections in one sweep over the layer: over the valid
-// elements of each whose key matches the prefix found so far.  Every position is valid for at most one of the two, so
-// one histogram of 512 bins (selection * 256 + digit) serves both.  A block takes whole rows, four columns per thread
-// and step when the row length is a multiple of four (16-byte loads of w and grad, 4-byte loads of the mask).
-template <bool LAST>  // the last sweep (pass 3) also fills the lists; the others keep their smaller code
-__global__ void __launch_bounds__(kThreads, 8) hist_kernel(const float* w, const uint8_t* mask, const float* grad, const int* row_count, int out_f, int in_f,
-                            int pass, SelectState* st, uint2* list, unsigned int cap) {
-    __shared__ unsigned int h[512];
-    __shared__ int list_full[2];
-    if (threadIdx.x < 2) list_full[threadIdx.x] = 0;
-    for (int b = threadIdx.x; b < 512; b += blockDim.x) h[b] = 0;
-    __syncthreads();
-    const bool on0 = st[0].want != 0, on1 = st[1].want != 0;
-    if (on0 || on1) {
-        const unsigned int prefix0 = st[0].prefix, pmask0 = st[0].prefix_mask, prefix1 = st[1].prefix, pmask1 = st[1].prefix_mask;
-        const int shift = 24 - 8 * pass;
-        auto one = [&](bool inside, uint8_t m, float wv, float gv, size_t pos) {  // every lane of the warp calls it the same number of times
-            bool take = false;
-            unsigned int bin = 0;
-            if (inside) {
-                const unsigned int key = m ? mag_bits(wv) : ~mag_bits(gv);
-                take = m ? (on0 && (key & pmask0) == prefix0) : (on1 && (key & pmask1) == prefix1);
-                bin = (m ? 0u : 256u) + ((key >> shift) & 255u);
-                if (LAST && take) {  // the last sweep lists what it counts, while the list has room
-                    const int sel = m ? 0 : 1;
-                    if (!list_full[sel]) {
-                        const unsigned int at = atomicAdd(&st[sel].listed, 1u);
-                        if (at < cap) list[(size_t)sel * cap + at] = make_uint2(key, (unsigned int)pos);
-                        else list_full[sel] = 1;
-                    }
-                }
+        for (int e = 0; e < kPer; ++e) {
+            if (!found && want <= (unsigned long long)seen + v[e]) {
+                out = Pick{(unsigned int)(kPer * t + e), seen, v[e]};
+                found = true;
             }
-            // The top digit falls into a handful of bins (aggregate per warp); the later digits of the few elements that
-            // still match the prefix spread out, and a plain atomic is cheaper there.
-            if (pass == 0) hist_add(h, take, bin);
-            else if (take) atomicAdd(&h[bin], 1u);
-        };
-        for (int r = blockIdx.x; r < out_f; r += gridDim.x) {
-            if (row_count[r] == 0) continue;  // a neuron without weights is in neither pool
-            const size_t base = (size_t)r * in_f;
-            if ((in_f & 3) == 0) {
-                const uchar4* m4 = reinterpret_cast<const uchar4*>(mask + base);
-                const float4* w4 = reinterpret_cast<const float4*>(w + base);
-                const float4* g4 = reinterpret_cast<const float4*>(grad + base);
-                const int n4 = in_f >> 2;
-                for (int v0 = 0; v0 < n4; v0 += blockDim.x) {
-                    const int v = v0 + threadIdx.x;
-                    const bool inside = v < n4;
-                    uchar4 m = make_uchar4(0, 0, 0, 0);
-                    float4 wv = make_float4(0.f, 0.f, 0.f, 0.f), gv = wv;
-                    if (inside) {  // all three at once: a load that waited for the mask would cost a second trip to memory
-                        m = m4[v];
-                        wv = w4[v];
-                        gv = g4[v];
-                    }
-                    one(inside, m.x, wv.x, gv.x, base + 4 * (size_t)v);
-                    one(inside, m.y, wv.y, gv.y, base + 4 * (size_t)v + 1);
-                    one(inside, m.z, wv.z, gv.z, base + 4 * (size_t)v + 2);
-                    one(inside, m.w, wv.w, gv.w, base + 4 * (size_t)v + 3);
-                }
-            } else {
-                for (int c0 = 0; c0 < in_f; c0 += blockDim.x) {
-                    const int c = c0 + threadIdx.x;
-                    const bool inside = c < in_f;
-                    const uint8_t m = inside ? mask[base + c] : 0;
-                    one(inside, m, inside && m ? w[base + c] : 0.f, inside && !m ? grad[base + c] : 0.f, base + c);
-                }
+            if (!found) seen += v[e];
+        }
+    }
+    __syncthreads();
+    return out;
+}
+
+// Called by the block of a sweep whose counts arrive last: both selections take their next digit from the histograms,
+// which are cleared for the next sweep.
+__device__ void narrow(State* st, bool first, long long K, int in_f, unsigned int cap) {
+    __shared__ unsigned int part[kThreads / 32];
+    __shared__ Pick pick;
+    __shared__ Select q[2];
+    constexpr int kPer = kBins / kThreads;
+    const int t = threadIdx.x;
+    uint4 v[2][kPer / 4];  // both histograms and the totals are on their way together: one trip to L2
+#pragma unroll
+    for (int s = 0; s < 2; ++s)
+#pragma unroll
+        for (int i = 0; i < kPer / 4; ++i) v[s][i] = __ldcg(reinterpret_cast<const uint4*>(st->hist[s]) + t * (kPer / 4) + i);
+    if (t == 0) {
+        if (first) {
+            const unsigned long long act = __ldcg(&st->active_total);
+            const unsigned long long inact = (unsigned long long)__ldcg(&st->live) * in_f - act;
+            unsigned long long kk = K < 0 ? 0ull : (unsigned long long)K;
+            kk = kk > act ? act : kk;
+            kk = kk > inact ? inact : kk;
+            for (int s = 0; s < 2; ++s) {
+                Select z{};
+                z.want = kk, z.on = kk != 0, z.shift = kAllBits;
+                z.count = (unsigned int)(s ? inact : act);  // at most 2^31
+                q[s] = z;
+            }
+        } else {
+            for (int s = 0; s < 2; ++s) {
+                q[s] = st->sel[s];
+                q[s].listed = __ldcg(&st->sel[s].listed);
             }
         }
     }
     __syncthreads();
-    for (int b = threadIdx.x; b < 512; b += blockDim.x)
-        if (h[b]) atomicAdd(&st[b >> 8].hist[b & 255], h[b]);
-    // The block whose counts arrive last narrows both selections to their bins (no separate launch, nobody waits).
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+        const int digit = q[s].shift < kDigit ? q[s].shift : kDigit;
+        if (q[s].on && digit > 0) {
+            unsigned int bins[kPer];
+#pragma unroll
+            for (int i = 0; i < kPer / 4; ++i) bins[4 * i] = v[s][i].x, bins[4 * i + 1] = v[s][i].y, bins[4 * i + 2] = v[s][i].z, bins[4 * i + 3] = v[s][i].w;
+            const Pick p = block_pick<kThreads>(q[s].want, bins, part, pick);
+            if (t == 0) {
+                q[s].prefix = (q[s].prefix << digit) | p.bin;
+                q[s].shift -= digit;
+                q[s].want -= p.below;
+                q[s].count = p.count;
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < kPer / 4; ++i) reinterpret_cast<uint4*>(st->hist[s])[t * (kPer / 4) + i] = make_uint4(0u, 0u, 0u, 0u);
+        __syncthreads();
+    }
+    if (t < 2) st->sel[t] = q[t];
+    if (t == 0) st->listable = (!q[0].on || q[0].count <= cap) && (!q[1].on || q[1].count <= cap);
+}
+
+// True in every thread of the block of this launch that gets here last; everything the other blocks wrote is visible.
+__device__ bool last_block(int* done) {
     __shared__ bool last;
     __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) last = atomicAdd(&st[0].blocks_done, 1u) == gridDim.x - 1;
-    __syncthreads();
-    if (last) {
-        __threadfence();
-        if (threadIdx.x < 64) pick_bin(pass, st + (threadIdx.x >> 5));
-        if (LAST) {  // both cuts are final
-            __syncthreads();
-            find_last_tie(st, list, cap);
-            __syncthreads();
-            find_last_tie(st + 1, list + cap, cap);
-        }
-        if (threadIdx.x == 0) st[0].blocks_done = 0;
+    if (threadIdx.x == 0) {
+        last = atomicAdd(done, 1) == (int)gridDim.x - 1;
+        if (last) *done = 0, __threadfence();
     }
+    __syncthreads();
+    return last;
 }
 
-// A thread's run of 16 consecutive positions from `base`: kind (0: in neither pool, 1: active weight, 2: inactive position
-// of a live neuron) and key of each.  When the run lies inside one row and the arrays allow 16-byte loads it takes one
-// load of the 16 mask bytes and four 16-byte loads each of the weights and the gradients, all requested together.
-__device__ __forceinline__ void load_run16(const float* w, const uint8_t* mask, const float* grad, const int* row_count, int in_f,
-                                           long long n, long long base, bool vec_ok, unsigned int (&keys)[16], uint8_t (&kind)[16]) {
-    if (vec_ok && base + 16 <= n) {
-        // Everything is requested at once: a load that waited for the mask would cost a second trip to memory.
-        const uint4 m16 = *reinterpret_cast<const uint4*>(mask + base);
-        float4 w16[4], g16[4];
-#pragma unroll
-        for (int g = 0; g < 4; ++g) {
-            w16[g] = *reinterpret_cast<const float4*>(w + base + 4 * g);
-            g16[g] = *reinterpret_cast<const float4*>(grad + base + 4 * g);
+// A sweep over the layer that counts the next digit of both selections' open elements; a block takes whole rows.  The
+// first sweep also counts the rows' weights (FIRST; whether a position of the gradient pool counts depends on whether
+// its row has any).  Later ones run only for layers with so many equal keys that a digit's open elements exceed the lists.
+//
+// Bound by memory: 9 bytes per entry, 4.4 TB/s on 4096 x 4096.  A thread has mask, weights and gradients of four chunks in
+// flight, of one row or of two or four short ones (3072 x 768: 21 us with one row at a time, 17 with four).  12-bit digits: a first digit of 8 exponent and 4 mantissa bits leaves about 1 % of the elements open, few
+// enough to list them in the next sweep instead of sweeping again for every digit.
+template <int VEC, int ROWS, bool FIRST>
+__global__ void __launch_bounds__(kThreads, 4) sweep_kernel(const float* w, const uint8_t* mask, const float* grad, int* row_count, int out_f,
+                                                         int in_f, long long K, unsigned int cap, State* st) {
+    extern __shared__ unsigned int h[];  // [2][kBins]
+    __shared__ int part[2][ROWS][kThreads / 32];
+    constexpr int kAhead = (VEC == 4 ? 4 : 8) / ROWS;  // chunks of each row
+    const int t = threadIdx.x;
+    for (int b = t; b < 2 * kBins; b += kThreads) h[b] = 0;
+    int shift[2] = {kAllBits, kAllBits}, digit[2] = {kDigit, kDigit};
+    unsigned long long prefix[2] = {0, 0};
+    bool on[2] = {true, true};
+    if (!FIRST) {
+        for (int s = 0; s < 2; ++s) {
+            prefix[s] = st->sel[s].prefix, shift[s] = st->sel[s].shift, on[s] = st->sel[s].on != 0;
+            digit[s] = shift[s] < kDigit ? shift[s] : kDigit;
         }
-        const unsigned int mw[4] = {m16.x, m16.y, m16.z, m16.w};
-        const bool live = row_count[(unsigned int)((unsigned long long)base / (unsigned int)in_f)] != 0;
+    }
+    __syncthreads();
+    unsigned long long total = 0;
+    int live = 0, k = 0, slot = 0;
+    auto count = [&](const Cols<VEC>& c, bool in, int col, size_t base) {
 #pragma unroll
-        for (int g = 0; g < 4; ++g) {
-            const unsigned int nz = __vcmpne4(mw[g], 0u);  // 0xff per nonzero mask byte
-            const float4 wv = w16[g], gv = g16[g];
-            const float we[4] = {wv.x, wv.y, wv.z, wv.w}, ge[4] = {gv.x, gv.y, gv.z, gv.w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const bool on = ((nz >> (8 * e)) & 1u) != 0u;
-                kind[4 * g + e] = on ? 1 : live ? 2 : 0;
-                keys[4 * g + e] = on ? mag_bits(we[e]) : live ? ~mag_bits(ge[e]) : 0u;
+        for (int e = 0; e < VEC; ++e) {
+            if (!in) continue;
+            const int s = c.on(e) ? 0 : 1;
+            const unsigned int key = s ? grad_key(c.g(e)) : weight_key(c.w(e));
+            if (FIRST) {
+                atomicAdd(&h[s * kBins + (key >> (kKeyBits - kDigit))], 1u);
+            } else if (on[s]) {
+                const unsigned int pos = (unsigned int)(base + col + e);
+                if (composite_top(key, pos, shift[s]) == prefix[s])
+                    atomicAdd(&h[s * kBins + (int)(composite_top(key, pos, shift[s] - digit[s]) & ((1u << digit[s]) - 1u))], 1u);
             }
         }
-        return;
-    }
+    };
+    for (long long r0 = blockIdx.x; r0 < out_f; r0 += (long long)ROWS * gridDim.x) {
+        Cols<VEC> c[ROWS][kAhead];
 #pragma unroll
-    for (int e = 0; e < 16; ++e) {
-        kind[e] = 0, keys[e] = 0;
-        const long long p = base + e;
-        if (p < n) {
-            if (mask[p]) kind[e] = 1, keys[e] = mag_bits(w[p]);
-            else if (row_count[(unsigned int)((unsigned long long)p / (unsigned int)in_f)] != 0) kind[e] = 2, keys[e] = ~mag_bits(grad[p]);
-        }
-    }
-}
-
-// After the four passes prefix is the key of the cut and `want` of the elements equal to it are taken, the first ones
-// in position order.  Per chunk of kChunk positions and per selection: how many equal the cut key.
-__global__ void tie_count_kernel(const float* w, const uint8_t* mask, const float* grad, const int* row_count, int in_f,
-                                 long long n, const SelectState* st, unsigned int* chunk_ties, int n_chunks, bool vec_ok) {
-    __shared__ unsigned int s[2];
-    if (st[0].listed_all && st[1].listed_all) return;  // the marking will not ask for tie counts
-    if (threadIdx.x < 2) s[threadIdx.x] = 0;
-    __syncthreads();
-    const long long base = (long long)blockIdx.x * kChunk + (long long)threadIdx.x * 16;
-    const bool on0 = st[0].want != 0, on1 = st[1].want != 0;
-    const unsigned int cut0 = st[0].prefix, cut1 = st[1].prefix;
-    unsigned int c0 = 0, c1 = 0;
-    unsigned int keys[16];
-    uint8_t kind[16];
-    load_run16(w, mask, grad, row_count, in_f, n, base, vec_ok, keys, kind);
+        for (int j = 0; j < ROWS; ++j) {
+            const long long r = r0 + (long long)j * gridDim.x;
 #pragma unroll
-    for (int e = 0; e < 16; ++e) {
-        c0 += (kind[e] == 1 && on0 && keys[e] == cut0) ? 1u : 0u;
-        c1 += (kind[e] == 2 && on1 && keys[e] == cut1) ? 1u : 0u;
-    }
-    if (c0) atomicAdd(&s[0], c0);
-    if (c1) atomicAdd(&s[1], c1);
-    __syncthreads();
-    if (threadIdx.x < 2) chunk_ties[(size_t)threadIdx.x * n_chunks + blockIdx.x] = s[threadIdx.x];
-}
-
-// One block per selection: exclusive prefix sum of its per-chunk tie counts, in place.
-__global__ void chunk_scan_kernel(unsigned int* chunk_ties_both, int n_chunks, const SelectState* st) {
-    if (st[0].listed_all && st[1].listed_all) return;
-    unsigned int* chunk_ties = chunk_ties_both + (size_t)blockIdx.x * n_chunks;
-    __shared__ unsigned long long warp_tot[kThreads / 32];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    // A thread takes 16 consecutive chunks at a time (the block 4096): their sum is scanned over the block with shuffles
-    // and one count per warp, then the thread walks its chunks.
-    unsigned long long carry = 0;
-    for (int c0 = 0; c0 < n_chunks; c0 += 16 * kThreads) {
-        const int first = c0 + 16 * threadIdx.x;
-        unsigned int v[16];
-        unsigned long long mine = 0;
-#pragma unroll
-        for (int e = 0; e < 16; ++e) v[e] = first + e < n_chunks ? chunk_ties[first + e] : 0u, mine += v[e];
-        unsigned long long incl = mine;
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const unsigned long long up = __shfl_up_sync(0xffffffffu, incl, off);
-            if (lane >= off) incl += up;
-        }
-        if (lane == 31) warp_tot[wid] = incl;
-        __syncthreads();
-        unsigned long long before = carry + incl - mine, total = 0;
-#pragma unroll
-        for (int i = 0; i < kThreads / 32; ++i) {
-            const unsigned long long p = warp_tot[i];
-            before += i < wid ? p : 0ull;
-            total += p;
-        }
-#pragma unroll
-        for (int e = 0; e < 16; ++e) {
-            if (first + e < n_chunks) chunk_ties[first + e] = (unsigned int)(before > 0xFFFFFFFFull ? 0xFFFFFFFFull : before);
-            before += v[e];
-        }
-        carry += total;
-        __syncthreads();  // warp_tot[] is rewritten by the next round
-    }
-}
-
-// drop[p] / grow_top[p] = 1 for the selected elements of the two selections: key below the cut, or equal to it and among
-// the first `want` in position order.
-__global__ void mark_kernel(const float* w, const uint8_t* mask, const float* grad, const int* row_count, int in_f, long long n,
-                            const SelectState* st, const unsigned int* chunk_ties, int n_chunks, uint8_t* drop,
-                            uint8_t* grow_top, bool vec_ok) {
-    __shared__ unsigned int part[2][kThreads];
-    const long long base = (long long)blockIdx.x * kChunk + (long long)threadIdx.x * 16;
-    const unsigned long long want0 = st[0].want, want1 = st[1].want;
-    const unsigned int cut0 = st[0].prefix, cut1 = st[1].prefix;
-    unsigned int keys[16];
-    uint8_t kind[16];  // 0: in neither pool, 1: active weight, 2: inactive position of a live neuron
-    unsigned int mine0 = 0, mine1 = 0;
-    load_run16(w, mask, grad, row_count, in_f, n, base, vec_ok, keys, kind);
-    unsigned int d16[4] = {0u, 0u, 0u, 0u}, g16[4] = {0u, 0u, 0u, 0u};  // the 16 flags of each kind, one byte each
-    if (st[0].listed_all && st[1].listed_all) {
-        // Both lists held every candidate of the last digit: a tie is taken up to a known position, nothing to rank.
-        const unsigned int last0 = st[0].last_tie, last1 = st[1].last_tie;
-#pragma unroll
-        for (int e = 0; e < 16; ++e) {
-            const unsigned int pos = (unsigned int)(base + e);
-            const unsigned int f0 = (kind[e] == 1 && want0 != 0 && (keys[e] < cut0 || (keys[e] == cut0 && pos <= last0))) ? 1u : 0u;
-            const unsigned int f1 = (kind[e] == 2 && want1 != 0 && (keys[e] < cut1 || (keys[e] == cut1 && pos <= last1))) ? 1u : 0u;
-            d16[e >> 2] |= f0 << (8 * (e & 3));
-            g16[e >> 2] |= f1 << (8 * (e & 3));
-        }
-    } else {
-#pragma unroll
-        for (int e = 0; e < 16; ++e) {
-            if (kind[e] == 1 && want0 != 0 && keys[e] == cut0) ++mine0;
-            if (kind[e] == 2 && want1 != 0 && keys[e] == cut1) ++mine1;
-        }
-        part[0][threadIdx.x] = mine0;
-        part[1][threadIdx.x] = mine1;
-        __syncthreads();
-        for (int off = 1; off < kThreads; off <<= 1) {
-            const unsigned int add0 = threadIdx.x >= off ? part[0][threadIdx.x - off] : 0u;
-            const unsigned int add1 = threadIdx.x >= off ? part[1][threadIdx.x - off] : 0u;
-            __syncthreads();
-            part[0][threadIdx.x] += add0;
-            part[1][threadIdx.x] += add1;
-            __syncthreads();
-        }
-        // ties of each selection before this thread's first element
-        unsigned long long rank0 = (unsigned long long)chunk_ties[blockIdx.x] + part[0][threadIdx.x] - mine0;
-        unsigned long long rank1 = (unsigned long long)chunk_ties[(size_t)n_chunks + blockIdx.x] + part[1][threadIdx.x] - mine1;
-#pragma unroll
-        for (int e = 0; e < 16; ++e) {
-            unsigned int f0 = 0, f1 = 0;
-            if (kind[e] == 1 && want0 != 0) {
-                if (keys[e] < cut0) f0 = 1;
-                else if (keys[e] == cut0) f0 = rank0++ < want0 ? 1 : 0;
-            } else if (kind[e] == 2 && want1 != 0) {
-                if (keys[e] < cut1) f1 = 1;
-                else if (keys[e] == cut1) f1 = rank1++ < want1 ? 1 : 0;
+            for (int u = 0; u < kAhead; ++u) {
+                const int col = (u * kThreads + t) * VEC;
+                c[j][u].load_mask(mask, (size_t)r * in_f + col, r < out_f && col < in_f);
+                c[j][u].load_values(w, grad, (size_t)r * in_f + col, r < out_f && col < in_f);
             }
-            d16[e >> 2] |= f0 << (8 * (e & 3));
-            g16[e >> 2] |= f1 << (8 * (e & 3));
         }
-    }
-    if (vec_ok && base + 16 <= n) {
-        *reinterpret_cast<uint4*>(drop + base) = make_uint4(d16[0], d16[1], d16[2], d16[3]);
-        *reinterpret_cast<uint4*>(grow_top + base) = make_uint4(g16[0], g16[1], g16[2], g16[3]);
-    } else {
+        if (FIRST) {
 #pragma unroll
-        for (int e = 0; e < 16; ++e) {
-            if (base + e >= n) continue;
-            drop[base + e] = (uint8_t)((d16[e >> 2] >> (8 * (e & 3))) & 1u);
-            grow_top[base + e] = (uint8_t)((g16[e >> 2] >> (8 * (e & 3))) & 1u);
+            for (int j = 0; j < ROWS; ++j) {
+                int mine = 0;
+#pragma unroll
+                for (int u = 0; u < kAhead; ++u) mine += c[j][u].count();
+                for (int col = (kAhead * kThreads + t) * VEC; ROWS == 1 && col < in_f; col += kThreads * VEC) {
+                    Cols<VEC> m;
+                    m.load_mask(mask, (size_t)r0 * in_f + col, true);
+                    mine += m.count();
+                }
+                mine = __reduce_add_sync(0xffffffffu, mine);
+                if ((t & 31) == 0) part[slot][j][t >> 5] = mine;
+            }
+            __syncthreads();  // one per step: the slots alternate
         }
+#pragma unroll
+        for (int j = 0; j < ROWS; ++j) {
+            const long long r = r0 + (long long)j * gridDim.x;
+            if (r >= out_f) continue;
+            int n = 0;
+            if (FIRST) {
+#pragma unroll
+                for (int i = 0; i < kThreads / 32; ++i) n += part[slot][j][i];
+                if (t == 0) row_count[r] = n, total += n, live += n > 0, k = max(k, n);
+            } else {
+                n = row_count[r];
+            }
+            if (n == 0) continue;  // a neuron without weights is in neither pool
+            const size_t base = (size_t)r * in_f;
+#pragma unroll
+            for (int u = 0; u < kAhead; ++u) count(c[j][u], (u * kThreads + t) * VEC < in_f, (u * kThreads + t) * VEC, base);
+            for (int c0 = kAhead * kThreads * VEC; ROWS == 1 && c0 < in_f; c0 += kAhead * kThreads * VEC) {
+#pragma unroll
+                for (int u = 0; u < kAhead; ++u) {
+                    const int col = c0 + (u * kThreads + t) * VEC;
+                    c[j][u].load_mask(mask, base + col, col < in_f);
+                    c[j][u].load_values(w, grad, base + col, col < in_f);
+                }
+#pragma unroll
+                for (int u = 0; u < kAhead; ++u) count(c[j][u], c0 + (u * kThreads + t) * VEC < in_f, c0 + (u * kThreads + t) * VEC, base);
+            }
+        }
+        slot ^= 1;
     }
+    __syncthreads();
+    for (int b = t; b < 2 * kBins; b += kThreads)
+        if (h[b]) atomicAdd(&st->hist[b / kBins][b % kBins], h[b]);
+    if (FIRST && t == 0 && live) {
+        atomicAdd(&st->active_total, total);
+        atomicAdd(&st->live, live);
+        atomicMax(&st->k, k);
+    }
+    if (last_block(&st->blocks_done)) narrow(st, FIRST, K, in_f, cap);
 }
 
-// Step 3: salient weights per neuron.
-__global__ void salient_kernel(const uint8_t* mask, const uint8_t* drop, const uint8_t* grow_top, int in_f, int* salient) {
-    __shared__ int s;
-    const int r = blockIdx.x;
-    if (threadIdx.x == 0) s = 0;
+// The last sweep: lists the open elements of both selections (key, position), counts their next digit, and counts per
+// row the weights that are salient whatever becomes of the open ones.  Listed elements are gathered in shared memory
+// and leave it together, so that the list's length is one global atomic per block and not one per element.
+template <int VEC, int ROWS>
+__global__ void __launch_bounds__(kThreads, 4) collect_kernel(const float* w, const uint8_t* mask, const float* grad, const int* row_count, int out_f,
+                                                           int in_f, unsigned int cap, uint2* list, int* salient, State* st) {
+    constexpr int kAhead = (VEC == 4 ? 4 : 8) / ROWS;  // chunks of each row
+    constexpr unsigned int kBuf = 1024;
+    __shared__ uint2 buf[2][kBuf];
+    __shared__ unsigned int n_buf[2], at_buf[2];
+    __shared__ int part[2][ROWS][kThreads / 32];
+    if (!st->listable) return;
+    const int t = threadIdx.x;
+    if (t < 2) n_buf[t] = 0;
+    // Both selections take the same number of elements, so both are on or off and have consumed the same digits.
+    const unsigned long long prefix0 = st->sel[0].prefix, prefix1 = st->sel[1].prefix;
+    const bool on = st->sel[0].on != 0;
+    const int shift = st->sel[0].shift, digit = shift < kDigit ? shift : kDigit;
+    // The cuts as the leading digits of a magnitude (a gradient's key is the complement of its bits).
+    const int key_shift = shift - kPosBits;
+    const unsigned int key_tops = key_shift > 0 ? 0x7FFFFFFFu >> key_shift : 0x7FFFFFFFu;
+    const unsigned int top_w = (unsigned int)prefix0, top_g = key_tops - (unsigned int)prefix1;
+    auto push = [&](bool is_w, unsigned int key, unsigned int pos) {
+        const int s = is_w ? 0 : 1;
+        atomicAdd(&st->hist[s][composite_top(key, pos, shift - digit) & ((1u << digit) - 1u)], 1u);
+        const unsigned int at = atomicAdd(&n_buf[s], 1u);
+        if (at < kBuf) {
+            buf[s][at] = make_uint2(key, pos);
+        } else {  // a row with more open elements than the buffer holds
+            const unsigned int g = atomicAdd(&st->sel[s].listed, 1u);
+            if (g < cap) list[(size_t)s * cap + g] = make_uint2(key, pos);
+        }
+    };
     __syncthreads();
-    int c = 0;
-    const size_t base = (size_t)r * in_f;
-    if ((in_f & 15) == 0 && (reinterpret_cast<uintptr_t>(mask) & 15u) == 0) {  // (the flag arrays are 256-byte aligned)
-        const uint4 *m16 = reinterpret_cast<const uint4*>(mask + base), *d16 = reinterpret_cast<const uint4*>(drop + base),
-                    *g16 = reinterpret_cast<const uint4*>(grow_top + base);
-        for (int v = threadIdx.x; v < (in_f >> 4); v += blockDim.x) {
-            const uint4 m = m16[v], d = d16[v], g = g16[v];
-            // a byte is salient if (mask set and not dropped) or among the top gradients
-            c += (__popc((__vcmpne4(m.x, 0u) & __vcmpeq4(d.x, 0u)) | __vcmpne4(g.x, 0u)) +
-                  __popc((__vcmpne4(m.y, 0u) & __vcmpeq4(d.y, 0u)) | __vcmpne4(g.y, 0u)) +
-                  __popc((__vcmpne4(m.z, 0u) & __vcmpeq4(d.z, 0u)) | __vcmpne4(g.z, 0u)) +
-                  __popc((__vcmpne4(m.w, 0u) & __vcmpeq4(d.w, 0u)) | __vcmpne4(g.w, 0u))) >> 3;
+    int slot = 0;
+    auto flush = [&]() {  // whole block
+        __syncthreads();
+        if (t < 2) {
+            const unsigned int n = n_buf[t] < kBuf ? n_buf[t] : kBuf;
+            at_buf[t] = n ? atomicAdd(&st->sel[t].listed, n) : 0u;
         }
-    } else if ((in_f & 3) == 0) {
-        const uchar4 *m4 = reinterpret_cast<const uchar4*>(mask + base), *d4 = reinterpret_cast<const uchar4*>(drop + base),
-                     *g4 = reinterpret_cast<const uchar4*>(grow_top + base);
-        for (int v = threadIdx.x; v < (in_f >> 2); v += blockDim.x) {
-            const uchar4 m = m4[v], d = d4[v], g = g4[v];
-            c += ((m.x && !d.x) || g.x) + ((m.y && !d.y) || g.y) + ((m.z && !d.z) || g.z) + ((m.w && !d.w) || g.w);
+        __syncthreads();
+#pragma unroll
+        for (int s = 0; s < 2; ++s)
+            for (unsigned int i = t; i < (n_buf[s] < kBuf ? n_buf[s] : kBuf); i += kThreads)
+                if (at_buf[s] + i < cap) list[(size_t)s * cap + at_buf[s] + i] = buf[s][i];
+        __syncthreads();
+        if (t < 2) n_buf[t] = 0;
+        __syncthreads();
+    };
+    for (long long r0 = blockIdx.x; r0 < out_f; r0 += (long long)ROWS * gridDim.x) {
+        int weights[ROWS], mine[ROWS];
+#pragma unroll
+        for (int j = 0; j < ROWS; ++j) {
+            const long long r = r0 + (long long)j * gridDim.x;
+            weights[j] = r < out_f ? row_count[r] : 0, mine[j] = 0;
         }
+        for (int c0 = 0; c0 < in_f; c0 += kAhead * kThreads * VEC) {
+            Cols<VEC> c[ROWS][kAhead];
+#pragma unroll
+            for (int j = 0; j < ROWS; ++j)
+#pragma unroll
+                for (int u = 0; u < kAhead; ++u) {
+                    const long long r = r0 + (long long)j * gridDim.x;
+                    const int col = c0 + (u * kThreads + t) * VEC;
+                    c[j][u].load_mask(mask, (size_t)r * in_f + col, r < out_f && col < in_f);
+                    c[j][u].load_values(w, grad, (size_t)r * in_f + col, r < out_f && col < in_f);
+                }
+#pragma unroll
+            for (int j = 0; j < ROWS; ++j)
+#pragma unroll
+            for (int u = 0; u < kAhead; ++u) {
+                const int col = c0 + (u * kThreads + t) * VEC;
+                // no weights: in neither pool; selections off: nothing is pruned and nothing grown
+                if (col >= in_f || weights[j] == 0 || !on) continue;
+                const size_t base = (size_t)(r0 + (long long)j * gridDim.x) * in_f;
+                if (key_shift >= 0) {
+                    // |v| against the selection's cut, both in the digits found so far.  In magnitudes a weight above its
+                    // cut stays and a gradient above its cut is taken: salient either way, so the two need no branches.
+                    bool open[VEC], any = false;
+#pragma unroll
+                    for (int e = 0; e < VEC; ++e) {
+                        const bool is_w = c[j][u].on(e);
+                        const unsigned int top = weight_key(is_w ? c[j][u].w(e) : c[j][u].g(e)) >> key_shift, at = is_w ? top_w : top_g;
+                        mine[j] += top > at;
+                        open[e] = top == at;
+                        any |= open[e];
+                    }
+                    if (any) {
+#pragma unroll
+                        for (int e = 0; e < VEC; ++e)
+                            if (open[e]) push(c[j][u].on(e), c[j][u].on(e) ? weight_key(c[j][u].w(e)) : grad_key(c[j][u].g(e)), (unsigned int)(base + col + e));
+                    }
+                } else {  // position digits: very many equal keys
+                    for (int e = 0; e < VEC; ++e) {
+                        const bool is_w = c[j][u].on(e);
+                        const unsigned int key = is_w ? weight_key(c[j][u].w(e)) : grad_key(c[j][u].g(e)), pos = (unsigned int)(base + col + e);
+                        const unsigned long long top = composite_top(key, pos, shift), at = is_w ? prefix0 : prefix1;
+                        mine[j] += is_w ? top > at : top < at;
+                        if (top == at) push(is_w, key, pos);
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < ROWS; ++j) {
+            const int n = __reduce_add_sync(0xffffffffu, mine[j]);
+            if ((t & 31) == 0) part[slot][j][t >> 5] = n;
+        }
+        __syncthreads();  // also completes these rows' entries
+        const long long mine_r = r0 + (long long)t * gridDim.x;
+        if (t < ROWS && mine_r < out_f) {
+            int n = 0;
+#pragma unroll
+            for (int i = 0; i < kThreads / 32; ++i) n += part[slot][t][i];
+            salient[mine_r] = on ? n : row_count[mine_r];
+        }
+        slot ^= 1;
+        const bool full = n_buf[0] > kBuf / 2 || n_buf[1] > kBuf / 2;
+        if (__syncthreads_or(full)) flush();
+    }
+    flush();
+    if (last_block(&st->blocks_done)) narrow(st, false, 0, in_f, cap);
+}
+
+// For lists in which one digit leaves too many elements open (very many equal keys): one more digit of both selections,
+// counted over the lists.
+__global__ void list_sweep_kernel(const uint2* list, unsigned int cap, int in_f, State* st) {
+    const unsigned int first = blockIdx.x * kThreads + threadIdx.x, step = gridDim.x * kThreads;
+    for (int s = 0; s < 2; ++s) {
+        const Select q = st->sel[s];
+        if (!q.on) continue;
+        const int digit = q.shift < kDigit ? q.shift : kDigit;
+        for (unsigned int i = first; i < q.listed; i += step) {
+            const uint2 e = list[(size_t)s * cap + i];
+            if (composite_top(e.x, e.y, q.shift) == q.prefix)
+                atomicAdd(&st->hist[s][composite_top(e.x, e.y, q.shift - digit) & ((1u << digit) - 1u)], 1u);
+        }
+    }
+    if (last_block(&st->blocks_done)) narrow(st, false, 0, in_f, cap);
+}
+
+// The `want`-th smallest composite (1-based) of `count` elements that the block's threads enumerate:
+// visit(f) calls f(key, pos) for each element, every element in exactly one thread.  Digits of 11 bits narrow the
+// elements down until there is at most one per thread; these are ranked against one another.
+constexpr unsigned int kRowBins = 2048;
+template <int T>
+struct SelectSmem {
+    alignas(16) unsigned int hist[kRowBins];
+    unsigned long long open[T];
+    unsigned long long result;
+    unsigned int part[T / 32], n;
+    Pick pick;
+};
+template <int T, typename Visit>
+__device__ unsigned long long block_select(unsigned int want, unsigned int count, Visit visit, SelectSmem<T>& sm) {
+    const int t = threadIdx.x;
+    unsigned long long prefix = 0;
+    int shift = kAllBits;
+    while (count > T && shift > 0) {
+        const int digit = shift < 11 ? shift : 11;
+        constexpr int kPer = kRowBins / T;
+#pragma unroll
+        for (int i = 0; i < kPer / 4; ++i) reinterpret_cast<uint4*>(sm.hist)[i * T + t] = make_uint4(0u, 0u, 0u, 0u);
+        __syncthreads();
+        if (shift == kAllBits) {
+            visit([&](unsigned int key, unsigned int) { atomicAdd(&sm.hist[key >> (kKeyBits - 11)], 1u); });
+        } else {
+            visit([&](unsigned int key, unsigned int pos) {
+                if (composite_top(key, pos, shift) == prefix)
+                    atomicAdd(&sm.hist[composite_top(key, pos, shift - digit) & ((1u << digit) - 1u)], 1u);
+            });
+        }
+        __syncthreads();
+        unsigned int bins[kPer];
+#pragma unroll
+        for (int i = 0; i < kPer / 4; ++i) {
+            const uint4 q = reinterpret_cast<const uint4*>(sm.hist)[t * (kPer / 4) + i];
+            bins[4 * i] = q.x, bins[4 * i + 1] = q.y, bins[4 * i + 2] = q.z, bins[4 * i + 3] = q.w;
+        }
+        const Pick p = block_pick<T>(want, bins, sm.part, sm.pick);
+        want -= p.below, count = p.count;
+        prefix = (prefix << digit) | p.bin;
+        shift -= digit;
+    }
+    if (t == 0) sm.n = 0;
+    __syncthreads();
+    auto list = [&](unsigned int key, unsigned int pos) {
+        const unsigned int at = atomicAdd(&sm.n, 1u);
+        if (at < T) sm.open[at] = composite(key, pos);
+    };
+    if (shift >= kPosBits) {  // the usual end: a key digit left few enough
+        const int key_shift = shift - kPosBits;
+        const unsigned int top = (unsigned int)prefix;
+        visit([&](unsigned int key, unsigned int pos) {
+            if (key >> key_shift == top) list(key, pos);
+        });
     } else {
-        for (int j = threadIdx.x; j < in_f; j += blockDim.x)
-            c += ((mask[base + j] && !drop[base + j]) || grow_top[base + j]) ? 1 : 0;
+        visit([&](unsigned int key, unsigned int pos) {
+            if (composite(key, pos) >> shift == prefix) list(key, pos);
+        });
     }
-    atomicAdd(&s, c);
     __syncthreads();
-    if (threadIdx.x == 0) salient[r] = s;
+    if ((unsigned int)t < count) {
+        const unsigned long long mine = sm.open[t];
+        unsigned int rank = 0;
+#pragma unroll 8
+        for (unsigned int i = 0; i < count; ++i) rank += sm.open[i] < mine;
+        if (rank == want - 1) sm.result = mine;
+    }
+    __syncthreads();
+    const unsigned long long result = sm.result;
+    __syncthreads();
+    return result;
 }
 
-// Steps 4 and 5 (single block): who is ablated, and the new fan-in.
-__global__ void ablate_kernel(const int* row_count, const int* salient, int out_f, int in_f, float gamma_sal, Scalars* sc,
-                              uint8_t* survives) {
-    __shared__ int after;
-    if (threadIdx.x == 0) after = 0;
+// Decides the listed elements: those below the cut's digits are taken, those above are not, and the last block finds the
+// cut among the few that are left.  Salient counts are completed on the way, then steps 4 and 5 (who is ablated, the new
+// fan-in) follow from them.
+__global__ void __launch_bounds__(kThreads) resolve_kernel(const uint2* list, unsigned int cap, uint2* ties, unsigned int ties_cap, const int* row_count,
+                                                           int* salient, uint8_t* survives, int out_f, int in_f, float gamma_sal, State* st) {
+    __shared__ SelectSmem<kThreads> sm;
+    __shared__ int part[2][kThreads / 32];
+    if (!st->listable) return;
+    for (int s = 0; s < 2; ++s)
+        if (st->sel[s].on && st->sel[s].count > ties_cap) return;  // another digit first (list_sweep_kernel)
+    const int t = threadIdx.x;
+    const unsigned int first = blockIdx.x * kThreads + t, step = gridDim.x * kThreads;
+    for (int s = 0; s < 2; ++s) {
+        if (!st->sel[s].on) continue;
+        const unsigned long long prefix = st->sel[s].prefix;
+        const int shift = st->sel[s].shift;
+        const unsigned int n = st->sel[s].listed;
+        for (unsigned int i = first; i < n; i += step) {
+            const uint2 e = list[(size_t)s * cap + i];
+            const unsigned long long top = composite_top(e.x, e.y, shift);
+            if (top == prefix) {
+                const unsigned int at = atomicAdd(&st->sel[s].listed_ties, 1u);
+                if (at < ties_cap) ties[(size_t)s * ties_cap + at] = e;
+            } else if ((s == 0) == (top > prefix)) {
+                atomicAdd(&salient[e.y / (unsigned int)in_f], 1);  // a weight that stays, a gradient that is taken
+            }
+        }
+    }
+    if (!last_block(&st->blocks_done)) return;
+    for (int s = 0; s < 2; ++s) {
+        const Select& q = st->sel[s];
+        if (!q.on) continue;
+        const unsigned int n = __ldcg(&q.listed_ties);
+        const uint2* mine = ties + (size_t)s * ties_cap;
+        const uint2 own = t < (int)n ? __ldcg(&mine[t]) : make_uint2(0u, 0u);
+        const unsigned long long cut = block_select<kThreads>((unsigned int)q.want, n, [&](auto f) {
+            if (t < (int)n) f(own.x, own.y);
+            for (unsigned int i = t + kThreads; i < n; i += kThreads) {
+                const uint2 e = __ldcg(&mine[i]);
+                f(e.x, e.y);
+            }
+        }, sm);
+        for (unsigned int i = t; i < n; i += kThreads) {
+            const uint2 e = __ldcg(&mine[i]);
+            if ((s == 0) == (composite(e.x, e.y) > cut)) atomicAdd(&salient[e.y / (unsigned int)in_f], 1);
+        }
+        if (t == 0) st->sel[s].cut = cut;
+        __syncthreads();
+    }
+    __threadfence();
     __syncthreads();
-    const double threshold = fmax(1.0, (double)gamma_sal * (double)sc->k);
+    // Steps 4 and 5.
+    const double threshold = fmax(1.0, (double)gamma_sal * (double)st->k);
     int mine = 0;
-    for (int r0 = threadIdx.x; r0 < out_f; r0 += 8 * blockDim.x) {  // eight rows' loads in flight: one block walks all rows
+    for (int r0 = t; r0 < out_f; r0 += 8 * kThreads) {  // eight rows' loads in flight: one block walks all rows
         int rc[8], sa[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
-            const int r = r0 + u * blockDim.x;
-            rc[u] = r < out_f ? row_count[r] : 0, sa[u] = r < out_f ? salient[r] : 0;
+            const int r = r0 + u * kThreads;
+            rc[u] = r < out_f ? row_count[r] : 0, sa[u] = r < out_f ? __ldcg(&salient[r]) : 0;
         }
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
-            const int r = r0 + u * blockDim.x;
+            const int r = r0 + u * kThreads;
             if (r < out_f) {
                 const bool live = rc[u] > 0 && !((double)sa[u] < threshold);
                 survives[r] = live ? 1 : 0;
@@ -561,328 +619,164 @@ __global__ void ablate_kernel(const int* row_count, const int* salient, int out_
             }
         }
     }
-    for (int off = 16; off > 0; off >>= 1) mine += __shfl_down_sync(0xffffffffu, mine, off);
-    if ((threadIdx.x & 31) == 0 && mine) atomicAdd(&after, mine);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        sc->live_after = after;
-        long long kn = after > 0 ? ((long long)sc->k * sc->live_before) / after : 0;
+    const int after = block_sum<kThreads>(mine, part, 0);
+    if (t == 0) {
+        long long kn = after > 0 ? ((long long)st->k * st->live) / after : 0;
         if (kn > in_f) kn = in_f;
-        sc->k_new = (int)kn;
+        st->k_new = (int)kn, st->live_after = after, st->done = 1;
     }
 }
 
-// Block-wide selection inside one row: the `m` smallest keys (ties to the smaller column) among the columns for which
-// `key_of` returns true.  Returns through shared memory the cut key and how many ties on it to take; `take(c, key)`
-// then answers for a column in increasing column order within the calling pattern below.
-struct RowCut {
-    unsigned int cut;
-    unsigned int ties;   // elements equal to the cut to take, the first ones in column order
-    int any;             // 0: nothing to select
-};
-
-// `count(prefix, prefix_mask, shift)` adds to hist[(key >> shift) & 255], with shared-memory atomics, every candidate of
-// the row whose key matches the prefix found so far.
-template <typename Count>
-__device__ void row_select(int m, Count count, unsigned int* hist /*256, shared*/, RowCut* out /*shared*/) {
-    __shared__ unsigned int prefix, pmask, want, warp_tot[kThreads / 32];
-    if (threadIdx.x == 0) prefix = 0, pmask = 0, want = (unsigned int)(m > 0 ? m : 0);
-    __syncthreads();
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int pass = 0; pass < 4 && m > 0; ++pass) {
-        for (int b = threadIdx.x; b < 256; b += blockDim.x) hist[b] = 0;
-        __syncthreads();
-        const int shift = 24 - 8 * pass;
-        count(prefix, pmask, shift);
-        __syncthreads();
-        // The bin that holds the `want`-th element, by the whole block (one bin per thread): the first bin whose running
-        // count reaches `want`, the last bin if none does.  A prefix count over the block (shuffles, then one count per
-        // warp); exactly one thread finds that the running count first reaches `want` in its bin.
-        {
-            const unsigned int h = hist[threadIdx.x], w0 = want;
-            unsigned int incl = h;
+// Steps 6 and 7 for one neuron per block: prune, then trim or regrow to k'.  A thread keeps the keys of its columns (rows of
+// up to COLS columns) in registers, so that the row is read once; longer rows (COLS = 0) are read again for every visit.
+//
+// 9 bytes read per entry, and of the outputs only what changes is written (a masked-off weight is 0 already, a kept one
+// keeps its value); bound by instruction issue as much as by memory, hence the one key per column: columns that cannot be
+// chosen carry kNoKey, above every key, and every later step is a compare (4096 x 4096: 105 us with 62-bit compares per
+// column, 73 with these).  The selection takes two visits of the row as a
+// rule: one 11-bit digit, then the few dozen elements left in its bin are ranked against one another.
+constexpr unsigned int kNoKey = 0xFFFFFFFFu;
+template <int VEC, int COLS, int T>
+__global__ void __launch_bounds__(T, (COLS > 2048 ? 1024 : 1536) / T) finalize_kernel(float* w, uint8_t* mask, const float* grad, const uint8_t* survives,
+                                                                              int in_f, const State* st) {
+    __shared__ SelectSmem<T> sm;
+    __shared__ int part[2][T / 32];
+    constexpr bool kCached = COLS > 0;
+    constexpr int kChunks = kCached ? COLS / (T * VEC) : 1;
+    const int r = blockIdx.x, t = threadIdx.x;
+    const size_t base = (size_t)r * in_f;
+    float* wr = w + base;
+    uint8_t* mr = mask + base;
+    const float* gr = grad + base;
+    Cols<VEC> c[kChunks];
+    if (kCached) {  // on the way while the flags below are read
 #pragma unroll
-            for (int off = 1; off < 32; off <<= 1) {
-                const unsigned int up = __shfl_up_sync(0xffffffffu, incl, off);
-                if (lane >= off) incl += up;
-            }
-            if (lane == 31) warp_tot[wid] = incl;
-            __syncthreads();
-            unsigned int before = 0, total = 0;
-#pragma unroll
-            for (int i = 0; i < kThreads / 32; ++i) {
-                const unsigned int p = warp_tot[i];
-                before += i < wid ? p : 0u;
-                total += p;
-            }
-            const unsigned int excl = before + incl - h;
-            const bool here = excl < w0 && w0 <= excl + h;
-            const bool last_none = w0 > total && threadIdx.x == kThreads - 1;
-            __syncthreads();  // every thread has read `want`
-            if (here || last_none) {
-                want = w0 - excl;
-                prefix |= (unsigned int)threadIdx.x << shift;
-                pmask |= 255u << shift;
-            }
+        for (int u = 0; u < kChunks; ++u) {
+            const int col = (u * T + t) * VEC;
+            c[u].load_mask(mr, col, col < in_f);
+            c[u].load_values(wr, gr, col, col < in_f);
         }
-        __syncthreads();
     }
-    if (threadIdx.x == 0) out->cut = prefix, out->ties = want, out->any = m > 0 ? 1 : 0;
-    __syncthreads();
-}
-
-// Steps 6 and 7 for one neuron per block: prune, then trim or regrow to k'.  The row's keys for the selection that turns
-// out to be needed (magnitudes of the kept weights when trimming, complemented gradient magnitudes of the free positions
-// when regrowing) are put in shared memory once, next to a byte per column that says whether the column is kept, so
-// that every 32-bit key value stays usable.  CACHED = false reads the operands from global memory on every pass
-// instead (rows too long for shared memory).
-template <bool CACHED>
-__global__ void finalize_kernel(float* w, uint8_t* mask, const float* grad, const uint8_t* drop, const uint8_t* survives,
-                                int in_f, const Scalars* sc) {
-    extern __shared__ __align__(16) unsigned char row_smem[];  // CACHED: keys[in_f] (4 bytes each), then state[in_f] (1 byte each)
-    __shared__ unsigned int hist[256];
-    __shared__ RowCut cut;
-    __shared__ int kept_count;
-    __shared__ unsigned int part[kThreads / 32];
-    const int r = blockIdx.x;
-    float* wr = w + (size_t)r * in_f;
-    uint8_t* mr = mask + (size_t)r * in_f;
-    const float* gr = grad + (size_t)r * in_f;
-    const uint8_t* dr = drop + (size_t)r * in_f;
+    if (!st->done) return;
     if (!survives[r]) {  // ablated now or before: nothing left
-        for (int c = threadIdx.x; c < in_f; c += blockDim.x) wr[c] = 0.0f, mr[c] = 0;
+        for (int c = t * VEC; c < in_f; c += T * VEC) {
+            if (VEC == 4) *reinterpret_cast<float4*>(wr + c) = make_float4(0.f, 0.f, 0.f, 0.f), *reinterpret_cast<unsigned int*>(mr + c) = 0u;
+            else wr[c] = 0.0f, mr[c] = 0;
+        }
         return;
     }
-    unsigned int* keys = reinterpret_cast<unsigned int*>(row_smem);
-    uint8_t* state = row_smem + (size_t)in_f * 4;  // 1 = kept after step 6, 0 = free
-    const int k_new = sc->k_new;
-    if (threadIdx.x == 0) kept_count = 0;
-    __syncthreads();
-    int mine = 0;
-    for (int c = threadIdx.x; c < in_f; c += blockDim.x) {
-        const bool is_kept = mr[c] && !dr[c];
-        if (CACHED) state[c] = is_kept ? 1 : 0;
-        mine += is_kept ? 1 : 0;
-    }
-    atomicAdd(&kept_count, mine);
-    __syncthreads();
-    const int kept = kept_count;
-    const bool trim = kept > k_new;
-    const int m = trim ? kept - k_new : k_new - kept;
-    if (CACHED && m > 0) {
-        for (int c = threadIdx.x; c < in_f; c += blockDim.x) {
-            const bool candidate = trim ? state[c] != 0 : state[c] == 0;
-            keys[c] = candidate ? (trim ? mag_bits(wr[c]) : ~mag_bits(gr[c])) : 0u;
-        }
-        __syncthreads();
-    }
-    auto key_of = [&](int c, unsigned int& key) {
-        if (CACHED) {
-            key = keys[c];
-            return trim ? state[c] != 0 : state[c] == 0;
-        }
-        const bool is_kept = mr[c] && !dr[c];
-        key = trim ? mag_bits(wr[c]) : ~mag_bits(gr[c]);
-        return trim ? is_kept : !is_kept;
+    const int k_new = st->k_new;
+    const bool on0 = st->sel[0].on != 0;
+    const unsigned int cut_key = (unsigned int)(st->sel[0].cut >> kPosBits);
+    // Position of the last pruned weight of magnitude cut_key, as a column of this row.
+    const long long cut_col = (long long)(st->sel[0].cut & 0x7FFFFFFFull) - (long long)base;
+    // Kept after step 6: in the mask and not among the K smallest of the layer.
+    auto is_kept = [&](const Cols<VEC>& c, int e, int col) {
+        const unsigned int u = weight_key(c.w(e));
+        const bool dropped = u < cut_key || (u == cut_key && (long long)(col + e) <= cut_col);
+        return c.on(e) && !(on0 && dropped);
     };
-    // trim: the kept weights with the smallest magnitudes go; otherwise the free positions with the largest gradient
-    // magnitudes come
-    row_select(m, [&](unsigned int pre, unsigned int pm, int shift) {
-        for (int c = threadIdx.x; c < in_f; c += blockDim.x) {
-            unsigned int key;
-            if (key_of(c, key) && (key & pm) == pre) atomicAdd(&hist[(key >> shift) & 255u], 1u);
-        }
-    }, hist, &cut);
-    // Apply, walking the row in column order so that ties on the cut key go to the smaller columns: a tie's rank is
-    // the ties of the chunks before (carried by every thread), of the warps before in this chunk (one count per warp
-    // in shared memory) and of the lanes before in its warp (a ballot).
-    unsigned int carry = 0;
-    for (int c0 = 0; c0 < in_f; c0 += kThreads) {
-        const int c = c0 + threadIdx.x;
-        bool is_kept = false, candidate = false;
-        unsigned int key = 0;
-        if (c < in_f) {
-            is_kept = CACHED ? state[c] != 0 : (mr[c] && !dr[c]);
-            candidate = trim ? is_kept : !is_kept;
-            if (cut.any && candidate) key = CACHED ? keys[c] : (trim ? mag_bits(wr[c]) : ~mag_bits(gr[c]));
-        }
-        const unsigned int tie = (cut.any && candidate && key == cut.cut) ? 1u : 0u;
-        const unsigned int ties_in_warp = __ballot_sync(0xffffffffu, tie != 0);
-        const int wid = threadIdx.x >> 5, ln = threadIdx.x & 31;
-        if (ln == 0) part[wid] = (unsigned int)__popc(ties_in_warp);
-        __syncthreads();
-        unsigned int rank = carry + (unsigned int)__popc(ties_in_warp & ((1u << ln) - 1u)), in_chunk = 0;
+    unsigned int key[kChunks][VEC], kept_bits[kChunks];
+    int mine = 0;
+    if (kCached) {
 #pragma unroll
-        for (int i = 0; i < kThreads / 32; ++i) {
-            const unsigned int p = part[i];
-            rank += i < wid ? p : 0u;
-            in_chunk += p;
+        for (int u = 0; u < kChunks; ++u) {
+            const int col = (u * T + t) * VEC;
+            kept_bits[u] = 0;
+#pragma unroll
+            for (int e = 0; e < VEC; ++e) {
+                const bool kept = is_kept(c[u], e, col);
+                if (!kept && __float_as_uint(c[u].w(e)) != 0u) wr[col + e] = 0.0f;  // pruned, or free (a weight grown later starts at 0)
+                kept_bits[u] |= kept ? 1u << e : 0u;
+                key[u][e] = kept || col >= in_f ? kNoKey : grad_key(c[u].g(e));
+            }
+            mine += __popc(kept_bits[u]);
         }
-        if (c < in_f) {
-            const bool selected = cut.any && candidate && (key < cut.cut || (tie && rank < cut.ties));
-            bool on;
-            if (trim) on = is_kept && !selected;
-            else on = is_kept || selected;
-            if (!on || !is_kept) wr[c] = 0.0f;  // pruned, trimmed, free, or grown (starts at 0); a survivor keeps its value
-            mr[c] = on ? 1 : 0;
+    } else {
+        for (int col = t * VEC; col < in_f; col += T * VEC) {
+            Cols<VEC> v;
+            v.load_mask(mr, col, true);
+            v.load_values(wr, gr, col, true);
+#pragma unroll
+            for (int e = 0; e < VEC; ++e) mine += is_kept(v, e, col) ? 1 : 0;
         }
-        carry += in_chunk;
-        __syncthreads();  // part[] is rewritten by the next chunk
+    }
+    const int kept = block_sum<T>(mine, part, 0);
+    const bool trim = kept > k_new;
+    const int m = trim ? kept - k_new : k_new - kept;
+    if (kCached && trim) {  // the other keys: magnitudes of the kept weights
+#pragma unroll
+        for (int u = 0; u < kChunks; ++u)
+#pragma unroll
+            for (int e = 0; e < VEC; ++e) key[u][e] = (kept_bits[u] >> e) & 1u ? weight_key(wr[(u * T + t) * VEC + e]) : kNoKey;
+    }
+    // Trim: the kept weights with the smallest magnitudes go; otherwise the free positions with the largest gradient
+    // magnitudes come.  Ties go to the smaller column.
+    unsigned long long cut = 0;
+    if (m > 0) {
+        cut = block_select<T>((unsigned int)m, (unsigned int)(trim ? kept : in_f - kept), [&](auto f) {
+            if (kCached) {
+#pragma unroll
+                for (int u = 0; u < kChunks; ++u)
+#pragma unroll
+                    for (int e = 0; e < VEC; ++e)
+                        if (key[u][e] != kNoKey) f(key[u][e], (unsigned int)((u * T + t) * VEC + e));
+            } else {
+                for (int col = t * VEC; col < in_f; col += T * VEC) {
+                    Cols<VEC> v;
+                    v.load_mask(mr, col, true);
+                    v.load_values(wr, gr, col, true);
+#pragma unroll
+                    for (int e = 0; e < VEC; ++e)
+                        if (is_kept(v, e, col) == trim) f(trim ? weight_key(v.w(e)) : grad_key(v.g(e)), (unsigned int)(col + e));
+                }
+            }
+        }, sm);
+    }
+    const unsigned int row_key = (unsigned int)(cut >> kPosBits), row_col = (unsigned int)(cut & 0x7FFFFFFFull);
+    auto chosen = [&](unsigned int k, int col) { return m > 0 && (k < row_key || (k == row_key && (unsigned int)col <= row_col)); };
+    if (kCached) {
+#pragma unroll
+        for (int u = 0; u < kChunks; ++u) {
+            const int col = (u * T + t) * VEC;
+            if (col >= in_f) continue;
+            unsigned int out = 0;
+#pragma unroll
+            for (int e = 0; e < VEC; ++e) {
+                const bool flip = chosen(key[u][e], col + e);  // a kept one goes, a free one comes
+                if (trim && flip) wr[col + e] = 0.0f;
+                out |= (((kept_bits[u] >> e) & 1u) != 0u) != flip ? 1u << (8 * e) : 0u;
+            }
+            if (VEC == 4) *reinterpret_cast<unsigned int*>(mr + col) = out;
+            else mr[col] = (uint8_t)out;
+        }
+    } else {
+        for (int col = t * VEC; col < in_f; col += T * VEC) {
+            Cols<VEC> v;
+            v.load_mask(mr, col, true);
+            v.load_values(wr, gr, col, true);
+            unsigned int out = 0;
+#pragma unroll
+            for (int e = 0; e < VEC; ++e) {
+                const bool was = is_kept(v, e, col);
+                const bool on = was != (was == trim && chosen(trim ? weight_key(v.w(e)) : grad_key(v.g(e)), col + e));
+                if (!(on && was) && __float_as_uint(v.w(e)) != 0u) wr[col + e] = 0.0f;
+                out |= on ? 1u << (8 * e) : 0u;
+            }
+            if (VEC == 4) *reinterpret_cast<unsigned int*>(mr + col) = out;
+            else mr[col] = (uint8_t)out;
+        }
     }
 }
 
-// The same step for rows whose length is a multiple of 16, whose arrays start on 16-byte boundaries and whose keys fit
-// in shared memory: a thread owns runs of 16 consecutive columns, so the row costs four dependent trips to memory (the
-// neuron's flag; mask and pruning flags, 16 bytes each; the keys, 16-byte loads of only the groups that hold candidates;
-// the weights once more for the write-back) instead of one per 256 columns and array, ties are ranked with one block-wide
-// prefix count per 4096 columns, and mask and weights go back in whole 16-byte stores.
-__global__ void __launch_bounds__(kThreads, 8) finalize_runs_kernel(float* w, uint8_t* mask, const float* grad, const uint8_t* drop, const uint8_t* survives,
-                                     int in_f, const Scalars* sc) {
-    extern __shared__ __align__(16) unsigned char row_smem[];  // keys[in_f] (4 bytes each), then state[in_f] (1 byte each)
-    __shared__ unsigned int hist[256];
-    __shared__ RowCut cut;
-    __shared__ int kept_count;
-    __shared__ unsigned int warp_tot[kThreads / 32];
-    const int r = blockIdx.x, t = threadIdx.x, lane = t & 31, wid = t >> 5, n_runs = in_f >> 4;
-    float* wr = w + (size_t)r * in_f;
-    uint8_t* mr = mask + (size_t)r * in_f;
-    const float* gr = grad + (size_t)r * in_f;
-    const uint8_t* dr = drop + (size_t)r * in_f;
-    if (!survives[r]) {  // ablated now or before: nothing left
-        for (int j = t; j < n_runs; j += kThreads) {
-            *reinterpret_cast<uint4*>(mr + 16 * j) = make_uint4(0u, 0u, 0u, 0u);
-#pragma unroll
-            for (int g = 0; g < 4; ++g) *reinterpret_cast<float4*>(wr + 16 * j + 4 * g) = make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-        return;
-    }
-    unsigned int* keys = reinterpret_cast<unsigned int*>(row_smem);
-    uint8_t* state = row_smem + (size_t)in_f * 4;  // 1 = kept after step 6, 0 = free
-    const int k_new = sc->k_new;
-    if (t == 0) kept_count = 0;
-    __syncthreads();
-    int mine = 0;
-    for (int j = t; j < n_runs; j += kThreads) {
-        const uint4 m = *reinterpret_cast<const uint4*>(mr + 16 * j), d = *reinterpret_cast<const uint4*>(dr + 16 * j);
-        uint4 st;  // a byte per column: 1 where the mask is set and the weight was not pruned in step 6
-        st.x = __vcmpne4(m.x, 0u) & __vcmpeq4(d.x, 0u) & 0x01010101u;
-        st.y = __vcmpne4(m.y, 0u) & __vcmpeq4(d.y, 0u) & 0x01010101u;
-        st.z = __vcmpne4(m.z, 0u) & __vcmpeq4(d.z, 0u) & 0x01010101u;
-        st.w = __vcmpne4(m.w, 0u) & __vcmpeq4(d.w, 0u) & 0x01010101u;
-        mine += __popc(st.x) + __popc(st.y) + __popc(st.z) + __popc(st.w);
-        *reinterpret_cast<uint4*>(state + 16 * j) = st;
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) mine += __shfl_down_sync(0xffffffffu, mine, off);
-    if (lane == 0 && mine) atomicAdd(&kept_count, mine);
-    __syncthreads();
-    const int kept = kept_count;
-    const bool trim = kept > k_new;
-    const int m = trim ? kept - k_new : k_new - kept;
-    if (m > 0) {
-        const float* src = trim ? wr : gr;
-        const unsigned int flip = trim ? 0u : 0xFFFFFFFFu;  // regrowing: the complement, so that a larger gradient is a smaller key
-        for (int j = t; j < n_runs; j += kThreads) {
-            const uint4 st = *reinterpret_cast<const uint4*>(state + 16 * j);
-            const unsigned int sw[4] = {st.x, st.y, st.z, st.w};
-#pragma unroll
-            for (int g = 0; g < 4; ++g) {
-                const unsigned int cand = trim ? sw[g] : (sw[g] ^ 0x01010101u);
-                uint4 kq = make_uint4(0u, 0u, 0u, 0u);
-                if (cand != 0u) {
-                    const float4 v = *reinterpret_cast<const float4*>(src + 16 * j + 4 * g);
-                    kq.x = (cand & 0x00000001u) ? (mag_bits(v.x) ^ flip) : 0u;
-                    kq.y = (cand & 0x00000100u) ? (mag_bits(v.y) ^ flip) : 0u;
-                    kq.z = (cand & 0x00010000u) ? (mag_bits(v.z) ^ flip) : 0u;
-                    kq.w = (cand & 0x01000000u) ? (mag_bits(v.w) ^ flip) : 0u;
-                }
-                *reinterpret_cast<uint4*>(keys + 16 * j + 4 * g) = kq;
-            }
-        }
-        __syncthreads();
-    }
-    // Four columns per thread and step: one 16-byte read of the keys, one 4-byte read of the state bytes.
-    row_select(m, [&](unsigned int pre, unsigned int pm, int shift) {
-        const unsigned int flip_state = trim ? 0u : 0x01010101u;
-        for (int q = t; q < (in_f >> 2); q += kThreads) {
-            const unsigned int cand = reinterpret_cast<const unsigned int*>(state)[q] ^ flip_state;
-            if (cand == 0u) continue;
-            const uint4 kq = reinterpret_cast<const uint4*>(keys)[q];
-            if ((cand & 0x00000001u) && (kq.x & pm) == pre) atomicAdd(&hist[(kq.x >> shift) & 255u], 1u);
-            if ((cand & 0x00000100u) && (kq.y & pm) == pre) atomicAdd(&hist[(kq.y >> shift) & 255u], 1u);
-            if ((cand & 0x00010000u) && (kq.z & pm) == pre) atomicAdd(&hist[(kq.z >> shift) & 255u], 1u);
-            if ((cand & 0x01000000u) && (kq.w & pm) == pre) atomicAdd(&hist[(kq.w >> shift) & 255u], 1u);
-        }
-    }, hist, &cut);
-    // Apply in column order, so that ties on the cut key go to the smaller columns: a tie's rank is the ties of the
-    // 4096-column chunks before (carried by every thread), of the threads before in this chunk (a prefix count over the
-    // block) and of the columns before in the thread's own run.
-    const bool any = cut.any != 0;
-    const unsigned int cut_key = cut.cut, cut_ties = cut.ties;
-    unsigned int carry = 0;
-    for (int j0 = 0; j0 < n_runs; j0 += kThreads) {
-        const int j = j0 + t;
-        const bool have = j < n_runs;
-        uint4 st = make_uint4(0u, 0u, 0u, 0u);
-        float4 wv[4];
-        if (have) {
-            st = *reinterpret_cast<const uint4*>(state + 16 * j);
-#pragma unroll
-            for (int g = 0; g < 4; ++g) wv[g] = *reinterpret_cast<const float4*>(wr + 16 * j + 4 * g);  // in flight during the count
-        }
-        const unsigned int sw[4] = {st.x, st.y, st.z, st.w};
-        unsigned int my_ties = 0;
-        if (have && any) {
-#pragma unroll
-            for (int g = 0; g < 4; ++g) {
-                const uint4 kq = *reinterpret_cast<const uint4*>(keys + 16 * j + 4 * g);
-                const unsigned int cand = trim ? sw[g] : (sw[g] ^ 0x01010101u);
-                my_ties += ((cand & 0x00000001u) && kq.x == cut_key) + ((cand & 0x00000100u) && kq.y == cut_key) +
-                           ((cand & 0x00010000u) && kq.z == cut_key) + ((cand & 0x01000000u) && kq.w == cut_key);
-            }
-        }
-        unsigned int incl = my_ties;
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const unsigned int up = __shfl_up_sync(0xffffffffu, incl, off);
-            if (lane >= off) incl += up;
-        }
-        if (lane == 31) warp_tot[wid] = incl;
-        __syncthreads();
-        unsigned int rank = carry + incl - my_ties, in_chunk = 0;
-#pragma unroll
-        for (int i = 0; i < kThreads / 32; ++i) {
-            const unsigned int p = warp_tot[i];
-            rank += i < wid ? p : 0u;
-            in_chunk += p;
-        }
-        if (have) {
-            unsigned int mo[4];
-#pragma unroll
-            for (int g = 0; g < 4; ++g) {
-                uint4 kq = make_uint4(0u, 0u, 0u, 0u);
-                if (any) kq = *reinterpret_cast<const uint4*>(keys + 16 * j + 4 * g);
-                const unsigned int kk[4] = {kq.x, kq.y, kq.z, kq.w};
-                float we[4] = {wv[g].x, wv[g].y, wv[g].z, wv[g].w};
-                mo[g] = 0u;
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const bool is_kept = ((sw[g] >> (8 * e)) & 1u) != 0u;
-                    const bool candidate = trim ? is_kept : !is_kept;
-                    const bool tie = any && candidate && kk[e] == cut_key;
-                    bool selected = any && candidate && kk[e] < cut_key;
-                    if (tie) selected = rank++ < cut_ties;
-                    const bool on = trim ? (is_kept && !selected) : (is_kept || selected);
-                    if (!on || !is_kept) we[e] = 0.0f;  // pruned, trimmed, free, or grown (starts at 0); a survivor keeps its value
-                    mo[g] |= (on ? 1u : 0u) << (8 * e);
-                }
-                *reinterpret_cast<float4*>(wr + 16 * j + 4 * g) = make_float4(we[0], we[1], we[2], we[3]);
-            }
-            *reinterpret_cast<uint4*>(mr + 16 * j) = make_uint4(mo[0], mo[1], mo[2], mo[3]);
-        }
-        carry += in_chunk;
-        __syncthreads();  // warp_tot[] is rewritten by the next chunk
-    }
+// Rows of up to 1024 columns take blocks of 128 threads: more rows are on an SM at once to hide one another's barriers.
+struct Finalize { void (*kernel)(float*, uint8_t*, const float*, const uint8_t*, int, const State*); int threads; };
+template <int VEC>
+Finalize finalize_for(int in_f) {
+    if (in_f <= 1024) return {finalize_kernel<VEC, 1024, 128>, 128};
+    if (in_f <= 2048) return {finalize_kernel<VEC, 2048, 256>, 256};
+    if (in_f <= 4096) return {finalize_kernel<VEC, 4096, 256>, 256};
+    return {finalize_kernel<VEC, 0, 256>, 256};
 }
 
 size_t align_up(size_t v) { return (v + 255) & ~(size_t)255; }
@@ -891,17 +785,17 @@ struct Workspace {
     int* row_count;
     int* salient;
     uint8_t* survives;
-    uint8_t* drop;
-    uint8_t* grow_top;
-    unsigned int* chunk_ties;
-    uint2* list;            // 2 x list_capacity(n) (key, position) pairs
-    SelectState* state;
-    Scalars* scalars;
+    State* state;
+    uint2* list;            // 2 x cap open elements
+    uint2* ties;            // 2 x ties_cap
+    unsigned int cap, ties_cap;
     size_t bytes;
 };
 
+// Together the state and the lists take 2 bytes per entry of the layer: room for nearly an eighth of it per selection.
+// The elements that one more digit leaves open have room for 1 / 64.
 Workspace carve(void* base, int out_f, int in_f) {
-    const size_t n = (size_t)out_f * in_f, chunks = (n + kChunk - 1) / kChunk;
+    const size_t n = (size_t)out_f * in_f;
     size_t off = 0;
     auto take = [&](size_t b) {
         const size_t at = off;
@@ -909,104 +803,127 @@ Workspace carve(void* base, int out_f, int in_f) {
         return static_cast<char*>(base) + at;
     };
     Workspace w{};
+    w.cap = (unsigned int)std::max<int64_t>(1024, (2 * (int64_t)n - (int64_t)sizeof(State)) / 16);
+    w.ties_cap = (unsigned int)(n / 64 < 64 ? 64 : n / 64 > 32768 ? 32768 : n / 64);
     w.row_count = reinterpret_cast<int*>(take((size_t)out_f * 4));
     w.salient = reinterpret_cast<int*>(take((size_t)out_f * 4));
     w.survives = reinterpret_cast<uint8_t*>(take((size_t)out_f));
-    w.drop = reinterpret_cast<uint8_t*>(take(n));
-    w.grow_top = reinterpret_cast<uint8_t*>(take(n));
-    w.chunk_ties = reinterpret_cast<unsigned int*>(take(2 * chunks * 4));
-    w.list = reinterpret_cast<uint2*>(take(2 * (size_t)list_capacity((long long)n) * sizeof(uint2)));
-    w.state = reinterpret_cast<SelectState*>(take(2 * sizeof(SelectState)));
-    w.scalars = reinterpret_cast<Scalars*>(take(sizeof(Scalars)));
+    w.state = reinterpret_cast<State*>(take(sizeof(State)));
+    w.list = reinterpret_cast<uint2*>(take(2 * (size_t)w.cap * sizeof(uint2)));
+    w.ties = reinterpret_cast<uint2*>(take(2 * (size_t)w.ties_cap * sizeof(uint2)));
     w.bytes = off;
     return w;
 }
 
-// Step 3's two selections over the whole layer (the first is also step 6's pruning set), in shared sweeps.
-bool layer_select_both(const float* w, const uint8_t* mask, const float* grad, const Workspace& ws, int out_f, int in_f,
-                       long long n, cudaStream_t st) {
-    const int chunks = (int)((n + kChunk - 1) / kChunk);
-    const int hist_blocks = out_f < 1184 ? out_f : 1184;  // whole rows per block, 8 CTAs per SM at most
-    for (int pass = 0; pass < 4; ++pass) {
-        if (pass < 3)
-            hist_kernel<false><<<hist_blocks, kThreads, 0, st>>>(w, mask, grad, ws.row_count, out_f, in_f, pass, ws.state, ws.list,
-                                                                 list_capacity(n));
-        else
-            hist_kernel<true><<<hist_blocks, kThreads, 0, st>>>(w, mask, grad, ws.row_count, out_f, in_f, pass, ws.state, ws.list,
-                                                                list_capacity(n));
-    }
-    // 16-byte loads and stores of a thread's run of 16 positions: the run must lie inside one row, and the arrays (the
-    // workspace's flag arrays are 256-byte aligned) must start on 16-byte boundaries.
-    const bool vec_ok = (in_f % 16) == 0 && ((reinterpret_cast<uintptr_t>(w) | reinterpret_cast<uintptr_t>(grad) |
-                                               reinterpret_cast<uintptr_t>(mask)) & 15u) == 0;
-    tie_count_kernel<<<chunks, kThreads, 0, st>>>(w, mask, grad, ws.row_count, in_f, n, ws.state, ws.chunk_ties, chunks, vec_ok);
-    chunk_scan_kernel<<<2, kThreads, 0, st>>>(ws.chunk_ties, chunks, ws.state);
-    mark_kernel<<<chunks, kThreads, 0, st>>>(w, mask, grad, ws.row_count, in_f, n, ws.state, ws.chunk_ties, chunks, ws.drop,
-                                             ws.grow_top, vec_ok);
-    return cudaGetLastError() == cudaSuccess;
-}
-
 // ---- cfi_pack_device: the condensed arrays straight from device-resident w and mask -------------------------------
 
-// Single block: rank of every non-empty row among the non-empty rows, their number, the common fan-in, and whether the
-// fan-in really is common.  info = {n_active, k, constant (1/0)}.
-__global__ void pack_rows_kernel(const int* row_count, int out_f, int* row_rank, int* info) {
-    __shared__ unsigned int part[kThreads];
-    __shared__ unsigned int carry;
-    __shared__ int k_min, k_max;
-    if (threadIdx.x == 0) carry = 0, k_min = 0x7fffffff, k_max = 0;
-    __syncthreads();
-    for (int r0 = 0; r0 < out_f; r0 += kThreads) {
-        const int r = r0 + threadIdx.x;
-        const int cnt = r < out_f ? row_count[r] : 0;
-        const unsigned int live = cnt > 0 ? 1u : 0u;
-        if (live) atomicMin(&k_min, cnt), atomicMax(&k_max, cnt);
-        part[threadIdx.x] = live;
-        __syncthreads();
-        for (int off = 1; off < kThreads; off <<= 1) {
-            const unsigned int add = threadIdx.x >= off ? part[threadIdx.x - off] : 0u;
-            __syncthreads();
-            part[threadIdx.x] += add;
-            __syncthreads();
+struct PackInfo { int n_active, k, constant, blocks_done; };
+
+// A lane's kVec consecutive mask bytes as a bit set (bit e: column e is kept).
+template <int VEC>
+__device__ __forceinline__ unsigned int kept_set(const uint8_t* m, int col, int in_f) {
+    if (VEC == 1) return col < in_f && m[col] ? 1u : 0u;
+    unsigned int bits = 0;
+    if (col < in_f) {
+        const uint4 v = *reinterpret_cast<const uint4*>(m + col);
+        const unsigned int q[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            // one bit per nonzero byte, gathered from bits 0, 8, 16, 24 of the comparison
+            const unsigned int nz = __vcmpne4(q[i], 0u) & 0x08040201u;
+            bits |= ((nz | (nz >> 8) | (nz >> 16) | (nz >> 24)) & 0xFu) << (4 * i);
         }
-        if (r < out_f) row_rank[r] = live ? (int)(carry + part[threadIdx.x] - 1) : -1;
-        __syncthreads();
-        if (threadIdx.x == kThreads - 1) carry += part[kThreads - 1];
-        __syncthreads();
     }
-    if (threadIdx.x == 0) info[0] = (int)carry, info[1] = k_max, info[2] = (carry == 0 || k_min == k_max) ? 1 : 0;
+    return bits;
 }
 
-// One block per row: its kept entries in increasing column order to values / indices of its rank.
-__global__ void pack_fill_kernel(const float* w, const uint8_t* mask, const int* row_rank, int in_f, int k, float* values,
-                                 int32_t* indices, int32_t* active_rows) {
-    __shared__ unsigned int part[kThreads];
-    __shared__ unsigned int carry;
-    const int r = blockIdx.x, rank = row_rank[r];
-    if (rank < 0) return;
-    if (threadIdx.x == 0) carry = 0, active_rows[rank] = r;
+// One warp per row: its number of kept weights.  The block that finishes last ranks the non-empty rows and finds the
+// common fan-in.  (A row is one or two kilobytes of mask: a block per row spent its time on barriers.)
+template <int VEC>
+__global__ void __launch_bounds__(kThreads) pack_rows_kernel(const uint8_t* mask, int out_f, int in_f, int* row_count, int* row_rank, PackInfo* info) {
+    __shared__ int part[kThreads / 32], k_min, k_max;
+    const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+    const int64_t r = (int64_t)blockIdx.x * (kThreads / 32) + wid;
+    if (r < out_f) {
+        int n = 0;
+#pragma unroll 4
+        for (int col = lane * VEC; col < in_f; col += 32 * VEC) n += __popc(kept_set<VEC>(mask + (size_t)r * in_f, col, in_f));
+        n = __reduce_add_sync(0xffffffffu, n);
+        if (lane == 0) row_count[r] = n;
+    }
+    if (!last_block(&info->blocks_done)) return;
+    if (t == 0) k_min = 0x7fffffff, k_max = 0;
+    constexpr int kPer = 8;  // consecutive rows per thread and round
+    int before = 0, lo = 0x7fffffff, hi = 0;
+    for (int r0 = 0; r0 < out_f; r0 += kPer * kThreads) {
+        int cnt[kPer], live = 0;
+#pragma unroll
+        for (int e = 0; e < kPer; ++e) {
+            const int row = r0 + kPer * t + e;
+            cnt[e] = row < out_f ? __ldcg(&row_count[row]) : 0;
+            if (cnt[e]) ++live, lo = min(lo, cnt[e]), hi = max(hi, cnt[e]);
+        }
+        int incl = live;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const int up = __shfl_up_sync(0xffffffffu, incl, off);
+            if (lane >= off) incl += up;
+        }
+        __syncthreads();  // part[] of the round before has been read
+        if (lane == 31) part[wid] = incl;
+        __syncthreads();
+        int rank = before + incl - live;
+#pragma unroll
+        for (int i = 0; i < kThreads / 32; ++i) {
+            rank += i < wid ? part[i] : 0;
+            before += part[i];
+        }
+#pragma unroll
+        for (int e = 0; e < kPer; ++e) {
+            const int row = r0 + kPer * t + e;
+            if (row < out_f) row_rank[row] = cnt[e] ? rank++ : -1;
+        }
+    }
     __syncthreads();
+    lo = __reduce_min_sync(0xffffffffu, lo), hi = __reduce_max_sync(0xffffffffu, hi);
+    if (lane == 0) atomicMin(&k_min, lo), atomicMax(&k_max, hi);
+    __syncthreads();
+    if (t == 0) info->n_active = before, info->k = k_max, info->constant = (before == 0 || k_min == k_max) ? 1 : 0;
+}
+
+// One warp per row: its kept entries in increasing column order to values / indices of its rank.  A lane takes VEC
+// consecutive columns, their place follows from a prefix count over the warp.
+template <int VEC>
+__global__ void __launch_bounds__(kThreads) pack_fill_kernel(const float* w, const uint8_t* mask, const int* row_rank, int out_f, int in_f,
+                                                             const PackInfo* info, float* values, int32_t* indices, int32_t* active_rows) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t r = (int64_t)blockIdx.x * (kThreads / 32) + warp;
+    if (!info->constant || r >= out_f) return;
+    const int rank = row_rank[r];
+    if (rank < 0) return;
+    if (lane == 0) active_rows[rank] = (int32_t)r;
     const float* wr = w + (size_t)r * in_f;
     const uint8_t* mr = mask + (size_t)r * in_f;
-    for (int c0 = 0; c0 < in_f; c0 += kThreads) {
-        const int c = c0 + threadIdx.x;
-        const unsigned int kept = (c < in_f && mr[c]) ? 1u : 0u;
-        part[threadIdx.x] = kept;
-        __syncthreads();
-        for (int off = 1; off < kThreads; off <<= 1) {
-            const unsigned int add = threadIdx.x >= off ? part[threadIdx.x - off] : 0u;
-            __syncthreads();
-            part[threadIdx.x] += add;
-            __syncthreads();
+    size_t at0 = (size_t)rank * info->k;
+    unsigned int next = kept_set<VEC>(mr, lane * VEC, in_f);
+    for (int c0 = 0; c0 < in_f; c0 += 32 * VEC) {
+        unsigned int bits = next;
+        const int col = c0 + lane * VEC, mine = __popc(bits);
+        next = kept_set<VEC>(mr, col + 32 * VEC, in_f);  // in flight while this chunk is written
+        int incl = mine;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const int up = __shfl_up_sync(0xffffffffu, incl, off);
+            if (lane >= off) incl += up;
         }
-        if (kept) {
-            const size_t at = (size_t)rank * k + carry + part[threadIdx.x] - 1;
+        size_t at = at0 + (incl - mine);
+        while (bits) {
+            const int c = col + __ffs(bits) - 1;
+            bits &= bits - 1;
             values[at] = wr[c];
-            indices[at] = c;
+            indices[at++] = c;
         }
-        __syncthreads();
-        if (threadIdx.x == kThreads - 1) carry += part[kThreads - 1];
-        __syncthreads();
+        at0 += __shfl_sync(0xffffffffu, incl, 31);
     }
 }
 
@@ -1029,27 +946,63 @@ extern "C" cfi_status_t cfi_srigl_update(float* w, uint8_t* mask, const float* g
     const Workspace ws = carve(workspace, out_features, in_features);
     if (workspace_bytes < ws.bytes) return CFI_ERR_BUFFER_TOO_SMALL;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    const long long n = (long long)out_features * in_features;
-    row_count_kernel<<<out_features, kThreads, 0, st>>>(mask, out_features, in_features, ws.row_count);
-    setup_kernel<<<1, kThreads, 0, st>>>(ws.row_count, out_features, in_features, (long long)K, ws.scalars, ws.state);
-    if (!layer_select_both(w, mask, grad, ws, out_features, in_features, n, st)) return CFI_ERR_CUDA;
-    salient_kernel<<<out_features, kThreads, 0, st>>>(mask, ws.drop, ws.grow_top, in_features, ws.salient);
-    ablate_kernel<<<1, kThreads, 0, st>>>(ws.row_count, ws.salient, out_features, in_features, gamma_sal, ws.scalars, ws.survives);
-    const size_t row_bytes = (size_t)in_features * 5;  // keys and one state byte per column
-    const bool runs_ok = (in_features % 16) == 0 && ((reinterpret_cast<uintptr_t>(w) | reinterpret_cast<uintptr_t>(grad) |
-                                                         reinterpret_cast<uintptr_t>(mask)) & 15u) == 0;
-    if (row_bytes <= 40 * 1024 && runs_ok && in_features >= 2048)  // shorter rows leave most of a block's threads without a run
-        finalize_runs_kernel<<<out_features, kThreads, row_bytes, st>>>(w, mask, grad, ws.drop, ws.survives, in_features, ws.scalars);
-    else if (row_bytes <= 40 * 1024)
-        finalize_kernel<true><<<out_features, kThreads, row_bytes, st>>>(w, mask, grad, ws.drop, ws.survives, in_features, ws.scalars);
-    else
-        finalize_kernel<false><<<out_features, kThreads, 0, st>>>(w, mask, grad, ws.drop, ws.survives, in_features, ws.scalars);
-    Scalars host{};
-    if (cudaGetLastError() != cudaSuccess ||
-        cudaMemcpyAsync(&host, ws.scalars, sizeof(host), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaStreamSynchronize(st) != cudaSuccess) {
-        cudaGetLastError();
-        return CFI_ERR_CUDA;
+    const bool vec = (in_features & 3) == 0 && (((uintptr_t)w | (uintptr_t)grad) & 15) == 0 && ((uintptr_t)mask & 3) == 0;
+    const int blocks = std::min(out_features, 148 * 4);  // one wave, whole rows per block
+    const size_t hist_bytes = 2 * kBins * sizeof(unsigned int);
+    StateHead host{};
+    auto wait = [&]() {
+        const bool ok = cudaGetLastError() == cudaSuccess && cudaMemcpyAsync(&host, static_cast<StateHead*>(ws.state), sizeof(host), cudaMemcpyDeviceToHost, st) == cudaSuccess &&
+                        cudaStreamSynchronize(st) == cudaSuccess;
+        if (!ok) cudaGetLastError();
+        return ok;
+    };
+    // Short rows: several at a time, so that a thread has as many loads in flight as in a long one.
+    const int chunk_cols = kThreads * (vec ? 4 : 1), ahead = vec ? 4 : 8;
+    const int rows = in_features <= ahead / 4 * chunk_cols ? 4 : in_features <= ahead / 2 * chunk_cols ? 2 : 1;
+    auto sweep = [&](auto first) {
+        constexpr bool F = decltype(first)::value;
+        auto go = [&](auto kernel) {
+            kernel<<<blocks, kThreads, hist_bytes, st>>>(w, mask, grad, ws.row_count, out_features, in_features, K, ws.cap, ws.state);
+        };
+        if (vec) rows == 4 ? go(sweep_kernel<4, 4, F>) : rows == 2 ? go(sweep_kernel<4, 2, F>) : go(sweep_kernel<4, 1, F>);
+        else rows == 4 ? go(sweep_kernel<1, 4, F>) : rows == 2 ? go(sweep_kernel<1, 2, F>) : go(sweep_kernel<1, 1, F>);
+    };
+    auto collect = [&]() {
+        auto go = [&](auto kernel) {
+            kernel<<<blocks, kThreads, 0, st>>>(w, mask, grad, ws.row_count, out_features, in_features, ws.cap, ws.list, ws.salient, ws.state);
+        };
+        if (vec) rows == 4 ? go(collect_kernel<4, 4>) : rows == 2 ? go(collect_kernel<4, 2>) : go(collect_kernel<4, 1>);
+        else rows == 4 ? go(collect_kernel<1, 4>) : rows == 2 ? go(collect_kernel<1, 2>) : go(collect_kernel<1, 1>);
+    };
+    auto resolve_and_finalize = [&]() {
+        resolve_kernel<<<2 * 148, kThreads, 0, st>>>(ws.list, ws.cap, ws.ties, ws.ties_cap, ws.row_count, ws.salient, ws.survives, out_features, in_features,
+                                                 gamma_sal, ws.state);
+        const Finalize f = vec ? finalize_for<4>(in_features) : finalize_for<1>(in_features);
+        f.kernel<<<out_features, f.threads, 0, st>>>(w, mask, grad, ws.survives, in_features, ws.state);
+    };
+    // The usual layer needs one sweep for the first digit and one that lists what it leaves open; nothing waits in between.
+    // The later kernels return at once where that does not do, and the rare rest of the way is driven from here.
+    if (cudaMemsetAsync(ws.state, 0, sizeof(State), st) != cudaSuccess) return CFI_ERR_CUDA;
+    sweep(std::true_type{});
+    collect();
+    resolve_and_finalize();
+    if (!wait()) return CFI_ERR_CUDA;
+    if (!host.done) {
+        const bool listed = host.listable != 0;
+        for (int i = 0; i < 6 && !host.listable; ++i) {  // very many equal keys: digit by digit until the open elements fit the lists
+            sweep(std::false_type{});
+            if (!wait()) return CFI_ERR_CUDA;
+        }
+        if (!listed) {
+            collect();
+            if (!wait()) return CFI_ERR_CUDA;
+        }
+        for (int i = 0; i < 6 && ((host.sel[0].on && host.sel[0].count > ws.ties_cap) || (host.sel[1].on && host.sel[1].count > ws.ties_cap)); ++i) {
+            list_sweep_kernel<<<148, kThreads, 0, st>>>(ws.list, ws.cap, in_features, ws.state);
+            if (!wait()) return CFI_ERR_CUDA;
+        }
+        resolve_and_finalize();
+        if (!wait()) return CFI_ERR_CUDA;
     }
     *k_new = host.k_new;
     *n_active_new = host.live_after;
@@ -1067,24 +1020,28 @@ extern "C" cfi_status_t cfi_pack_device(const float* w_dense, const uint8_t* mas
     if (workspace_bytes < (size_t)out_features * 8 + 256) return CFI_ERR_BUFFER_TOO_SMALL;
     int* row_count = static_cast<int*>(workspace);
     int* row_rank = row_count + out_features;
-    int* info = row_rank + out_features;
+    PackInfo* info = reinterpret_cast<PackInfo*>(row_rank + out_features);
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    row_count_kernel<<<out_features, kThreads, 0, st>>>(mask, out_features, in_features, row_count);
-    pack_rows_kernel<<<1, kThreads, 0, st>>>(row_count, out_features, row_rank, info);
-    int host[3] = {0, 0, 0};
-    if (cudaGetLastError() != cudaSuccess || cudaMemcpyAsync(host, info, sizeof(host), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+    const bool vec = (in_features & 15) == 0 && ((uintptr_t)mask & 15) == 0;
+    const int blocks = (int)(((int64_t)out_features + kThreads / 32 - 1) / (kThreads / 32));
+    PackInfo host{};
+    if (cudaMemsetAsync(info, 0, sizeof(PackInfo), st) != cudaSuccess) {
+        cudaGetLastError();
+        return CFI_ERR_CUDA;
+    }
+    if (vec) pack_rows_kernel<16><<<blocks, kThreads, 0, st>>>(mask, out_features, in_features, row_count, row_rank, info);
+    else pack_rows_kernel<1><<<blocks, kThreads, 0, st>>>(mask, out_features, in_features, row_count, row_rank, info);
+    if (fill) {  // writes nothing where the fan-in is not constant
+        if (vec) pack_fill_kernel<16><<<blocks, kThreads, 0, st>>>(w_dense, mask, row_rank, out_features, in_features, info, values, indices, active_rows);
+        else pack_fill_kernel<1><<<blocks, kThreads, 0, st>>>(w_dense, mask, row_rank, out_features, in_features, info, values, indices, active_rows);
+    }
+    if (cudaGetLastError() != cudaSuccess || cudaMemcpyAsync(&host, info, sizeof(host), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess) {
         cudaGetLastError();
         return CFI_ERR_CUDA;
     }
-    if (!host[2]) return CFI_ERR_NOT_CONSTANT_FAN_IN;
-    *n_active = host[0];
-    *k = host[0] ? host[1] : 0;
-    if (!fill || host[0] == 0) return CFI_OK;
-    pack_fill_kernel<<<out_features, kThreads, 0, st>>>(w_dense, mask, row_rank, in_features, host[1], values, indices, active_rows);
-    if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess) {
-        cudaGetLastError();
-        return CFI_ERR_CUDA;
-    }
+    if (!host.constant) return CFI_ERR_NOT_CONSTANT_FAN_IN;
+    *n_active = host.n_active;
+    *k = host.n_active ? host.k : 0;
     return CFI_OK;
 }

@@ -91,6 +91,59 @@ def test_ties_with_and_without_room_in_the_candidate_list(levels):
     _compare(w, m, g, 9000, 0.3)
 
 
+# Both load widths (rows a multiple of four columns or not) at the ends of each number of rows per step and of each row
+# length that the per-neuron step keeps in registers, with distinct keys, with many equal ones and with all gradients
+# equal (then the lists of open elements overflow and further digits, of the position too, are counted first).
+@pytest.mark.parametrize("values", ["distinct", "coarse", "equal"])
+@pytest.mark.parametrize("out_f,in_f", [(61, 255), (700, 257), (33, 512), (20, 513), (40, 1020), (37, 1024), (19, 1028), (24, 2047), (23, 2048),
+                                        (18, 2049), (17, 4095), (16, 4096), (12, 4100), (9, 4101)])
+def test_row_lengths(out_f, in_f, values):
+    w, m, g = _layer(out_f, in_f, max(1, in_f // 9), out_f // 10, seed=out_f * 7 + in_f)
+    if values != "distinct":
+        w = (np.ceil(np.abs(w) * 8) / 8 * np.sign(w) * (m == 1)).astype(np.float32)
+        g = np.round(g).astype(np.float32) if values == "coarse" else np.ones_like(g)
+    _compare(w, m, g, int(0.25 * m.sum()), 0.3)
+
+
+def test_equal_keys_fill_the_lists():
+    """512 x 2048 in whose gradients 2 % of the positions tie at the cut: more than the ties have room for (16384) and fewer
+    than the lists (126976), so that the listed elements take further digits before they are decided."""
+    w, m, g = _layer(512, 2048, 200, 0, seed=5)
+    g = (np.abs(g) * 1e-3).astype(np.float32)
+    flat = np.random.default_rng(1).permutation(512 * 2048)[:24_000]
+    g.ravel()[flat] = 0.5
+    _compare(w, m, g, 9_000, 0.3)
+
+
+def test_unaligned_arrays():
+    """Arrays that start off a 16-byte boundary take the one-column loads; what comes out is the same."""
+    import torch
+    from paper_2305_02299_b200 import binding as cfi
+    w, m, g = _layer(37, 512, 50, 3, seed=8)
+    w_ref, m_ref, k_ref, _ = srigl_update(w, m, g, 300, float(np.float32(0.3)))
+    dev = []
+    for a in (w, m, g):
+        t = torch.empty(a.size + 1, dtype=torch.from_numpy(a).dtype, device="cuda")[1:].view(a.shape)
+        t.copy_(torch.from_numpy(a))
+        dev.append(t)
+    k_new, _ = cfi.cfi_srigl_update(*dev, 300, 0.3)
+    assert k_new == k_ref and np.array_equal(dev[1].cpu().numpy(), m_ref) and np.array_equal(dev[0].cpu().numpy(), w_ref)
+    v, ix, rows = cfi.cfi_pack_device(dev[0], dev[1])
+    vh, ih, rh = cfi.cfi_pack(w_ref, m_ref)
+    assert np.array_equal(v.cpu().numpy(), vh) and np.array_equal(ix.cpu().numpy(), ih) and np.array_equal(rows.cpu().numpy(), rh)
+
+
+@pytest.mark.parametrize("out_f,in_f", [(1, 16), (9, 512), (8, 528), (2049, 32), (5000, 1040), (3, 8192)])
+def test_pack_row_and_column_chunks(out_f, in_f):
+    """Rows around the eight of a block and the 2048 of a ranking round, columns around the 512 of a warp's step."""
+    import torch
+    from paper_2305_02299_b200 import binding as cfi
+    w, m, _ = _layer(out_f, in_f, max(1, in_f // 11), out_f // 3, seed=out_f)
+    v, ix, rows = cfi.cfi_pack_device(torch.from_numpy(w).cuda(), torch.from_numpy(m).cuda())
+    vh, ih, rh = cfi.cfi_pack(w, m)
+    assert np.array_equal(v.cpu().numpy(), vh) and np.array_equal(ix.cpu().numpy(), ih) and np.array_equal(rows.cpu().numpy(), rh)
+
+
 def test_workspace_and_argument_checks():
     import ctypes
     import torch
