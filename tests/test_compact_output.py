@@ -95,3 +95,35 @@ def test_compact_pair_on_device(dtype, B):
     st.close(); l1.close(); l2.close()
     err = np.max(np.abs(y.float().cpu().numpy().astype(np.float64) - y_full) / S)
     assert err <= TOL[dtype]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("d_in,d_hid,d_out,B", [(256, 411, 128, 25), (256, 411, 128, 24), (255, 409, 131, 130), (65, 72, 7, 300), (136, 1001, 520, 2600),
+                                                (131, 1024, 1030, 5000)])
+def test_odd_widths_in_a_bf16_stack(d_in, d_hid, d_out, B):
+    """Chains whose widths TMA cannot address as they are: odd inside, at the ends, or both; batches on both sides of the
+    switch to the padded dense copies, one tile and several per SM.  The second layer is compared with the oracle on what
+    the first one gave, computed layer by layer without the stack."""
+    import torch
+    from parity import oracle_layer, run_device, to_device, torch_dtype
+    L1 = inputs.make_layer(d_in, d_hid, max(1, d_in // 10), n_ablated=d_hid // 20, seed=d_in)
+    L2 = inputs.make_layer(d_hid, d_out, max(1, d_hid // 10), n_ablated=d_out // 20, seed=d_out)
+    x = inputs.make_x(B, d_in, seed=B)
+    layers = [cfi.cfi_create(*cfi.cfi_pack(L.w_dense, L.mask), L.bias, L.in_features, L.out_features, dtype="bf16", act=a) for L, a in ((L1, "gelu"), (L2, "none"))]
+    h = run_device(layers[0], x, "bf16", "auto")
+    y_ref, S = oracle_layer(L2, h, "bf16", "none")
+    st = cfi.cfi_stack_create(layers, B)
+    guard = 64
+    buf = torch.full((B * d_out + guard,), 7.0, device="cuda", dtype=torch_dtype("bf16"))
+    for _ in range(2):
+        cfi.cfi_stack_forward(st, to_device(x, "bf16"), buf[:B * d_out].view(B, d_out), B)
+    torch.cuda.synchronize()
+    assert all(cfi.cfi_device_status(l) == 0 for l in layers)
+    assert bool((buf[B * d_out:] == 7.0).all())
+    y = buf[:B * d_out].view(B, d_out).float().cpu().numpy()
+    st.close()
+    for l in layers:
+        l.close()
+    # Inside the chain an element of h whose sum falls on the other side of a rounding boundary moves by up to 2^-8 of
+    # itself: all of them together move y by at most 2^-8 of S.  On top, y's own rounding and the fp32 sums.
+    assert np.all(np.abs(y - y_ref) <= 2.0 ** -8 * (np.abs(y_ref) + S) + 1e-5 * S)
