@@ -122,10 +122,29 @@ def _dev_ptr(t) -> int:
     return t.data_ptr()
 
 
+# The current stream of the current device as an address.  torch.cuda.current_stream() builds a Stream object around it,
+# 3.4 of the 8 us that a small call takes on the host (768 -> 3072 at batch 1: 8.1 us a call with it, 4.5 without).
+_current_raw_stream = None
+
+
+def _raw_stream() -> int:
+    global _current_raw_stream
+    if _current_raw_stream is None:
+        import torch
+        torch.cuda.init()
+        get_stream, get_device = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+        if get_stream is None or get_device is None:
+            def _current_raw_stream_py():
+                return torch.cuda.current_stream().cuda_stream
+            _current_raw_stream = _current_raw_stream_py
+        else:
+            _current_raw_stream = lambda: get_stream(get_device())  # noqa: E731
+    return _current_raw_stream()
+
+
 def _stream_handle(stream) -> int:
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        return _raw_stream()
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
