@@ -123,8 +123,8 @@ __global__ void cfi_simple_kernel(DevLayer L, const VT* __restrict__ x, VT* __re
 }
 
 // ------------------------------------------------------------------------------------------------
-// CFI_VARIANT_SPLITK: small batch.  G lanes share one output row and split its k terms; the CTA's
-// x rows sit in shared memory as xs[column][BT] (+ one zero column for pad entries).
+// CFI_VARIANT_SPLITK: small batch.  G lanes share one output row and split its k terms; x sits in shared memory (+ one
+// zero column for pad entries).  The kernel below takes fp32 layers at batch 1, cfi_splitk_rows.cuh has the other cases.
 // ------------------------------------------------------------------------------------------------
 // Units a lane of the split-k kernel keeps in flight: 4, or 2 of the 48-byte units of fp32 values with 16-bit columns
 // (the same lanes per row, and so the same launch shapes, as 4 units of 4 entries would give).
@@ -225,27 +225,6 @@ template <> struct Chunk<__nv_bfloat16, true> {  // 8 weights + 8 uint16 columns
     __device__ __forceinline__ int col(int e) const { return col16(c, e); }
 };
 
-template <int BT>
-__device__ __forceinline__ void gather_fma(float (&acc)[BT], const float* xs, int col, float w) {
-    const float* p = xs + (size_t)col * BT;
-    if constexpr (BT == 1) {
-        acc[0] = fmaf(w, p[0], acc[0]);
-    } else if constexpr (BT == 2) {
-        const float2 v = *reinterpret_cast<const float2*>(p);
-        acc[0] = fmaf(w, v.x, acc[0]);
-        acc[1] = fmaf(w, v.y, acc[1]);
-    } else {
-#pragma unroll
-        for (int q = 0; q < BT / 4; ++q) {
-            const float4 v = *reinterpret_cast<const float4*>(p + 4 * q);
-            acc[4 * q + 0] = fmaf(w, v.x, acc[4 * q + 0]);
-            acc[4 * q + 1] = fmaf(w, v.y, acc[4 * q + 1]);
-            acc[4 * q + 2] = fmaf(w, v.z, acc[4 * q + 2]);
-            acc[4 * q + 3] = fmaf(w, v.w, acc[4 * q + 3]);
-        }
-    }
-}
-
 // Programmatic dependent launch.  Every forward kernel lets its successor in the stream start early
 // (pdl_launch_dependents at its top) and itself touches x and y only after pdl_wait, which returns once the
 // predecessor has completed and its writes are visible.  What a kernel does before pdl_wait (reading the
@@ -261,18 +240,17 @@ __device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
 
 // A lane keeps U units (16-byte vectors of weights with their indices) in flight in registers; the rest of the row is
 // on its way into L2.  XS = loads of x in flight per thread while staging (8 where few threads stage a long x).
-template <typename VT, bool I16, int BT, int G, int XS>
-__global__ void __launch_bounds__(512) cfi_splitk_kernel(DevLayer L, const VT* __restrict__ x, VT* __restrict__ y, int batch,
-                                  int rows_per_group) {
-    extern __shared__ __align__(16) float xs_f32[];  // [(in + 1)][BT]
+template <bool I16, int G, int XS>
+__global__ void __launch_bounds__(512) cfi_splitk_kernel(DevLayer L, const float* __restrict__ x, float* __restrict__ y, int rows_per_group) {
+    extern __shared__ __align__(16) float xs_f32[];  // [in + 1]
     float* xs = xs_f32;
-    using CK = Chunk<VT, I16>;
+    using VT = float;
+    using CK = Chunk<float, I16>;
     constexpr uint32_t kIdxBytes = I16 ? 2 : 4;
-    constexpr int U = splitk_units_in_flight(sizeof(VT) == 4, I16);
+    constexpr int U = splitk_units_in_flight(true, I16);
     pdl_launch_dependents();
     const int tid = threadIdx.x, nthr = blockDim.x;
-    const int b0 = blockIdx.y * BT;
-    const int nb = min(BT, batch - b0);
+    const int b0 = blockIdx.y;  // one batch row per CTA
     const int groups = nthr / G, g = tid / G, lg = tid % G;
     const int nvec = L.kp / CK::VEC;
     const bool dense_rows = L.identity_rows != 0;  // output row o is condensed row o: no look-up through slot[]
@@ -298,70 +276,50 @@ __global__ void __launch_bounds__(512) cfi_splitk_kernel(DevLayer L, const VT* _
     // into L2 reads nothing (L2 is where that kernel's writes land, so nothing stale can be kept), and a cold x is
     // then on chip when the wait returns.  The first CTAs of a batch tile ask, 16 KB per thread.
     if (blockIdx.x < 2 && ((size_t)L.in * sizeof(VT)) % 16 == 0) {
-        const size_t bytes = (size_t)nb * L.in * sizeof(VT), off = (size_t)tid << 14;
+        const size_t bytes = (size_t)L.in * sizeof(VT), off = (size_t)tid << 14;
         if (off < bytes)
             prefetch_l2(reinterpret_cast<const unsigned char*>(x + (size_t)b0 * L.in) + off, (uint32_t)min(bytes - off, (size_t)1 << 14));
     }
 
     pdl_wait();
-    // Stage the CTA's x rows, widened to fp32, transposed to [column][b].  Loads are issued kXStage at a time
-    // before their stores, so staging costs a few memory round trips, not one per element.
-    constexpr int kXStage = XS;
-    if (BT == 1 && sizeof(VT) == 4 && (L.in & 3) == 0) {
-        const float4* src = reinterpret_cast<const float4*>(reinterpret_cast<const float*>(x) + (size_t)b0 * L.in);
+    // Stage the CTA's row of x.  Loads are issued XS at a time before their stores, so staging costs a few memory round
+    // trips, not one per element.
+    if ((L.in & 3) == 0) {
+        const float4* src = reinterpret_cast<const float4*>(x + (size_t)b0 * L.in);
         const int n4 = L.in >> 2;
-        for (int c0 = tid; c0 < n4; c0 += nthr * kXStage) {
-            float4 v[kXStage];
+        for (int c0 = tid; c0 < n4; c0 += nthr * XS) {
+            float4 v[XS];
 #pragma unroll
-            for (int u = 0; u < kXStage; ++u)
+            for (int u = 0; u < XS; ++u)
                 if (c0 + u * nthr < n4) v[u] = __ldg(src + c0 + u * nthr);
 #pragma unroll
-            for (int u = 0; u < kXStage; ++u)
+            for (int u = 0; u < XS; ++u)
                 if (c0 + u * nthr < n4) reinterpret_cast<float4*>(xs)[c0 + u * nthr] = v[u];
         }
     } else {
-        // A thread takes kCols columns at a time: one load per column and batch row (each coalesced across the
-        // warp), all issued before the first store, then each column's BT values go to shared memory side by side.
-        constexpr int kCols = BT >= 8 ? 4 : BT >= 4 ? 4 : 8;
+        constexpr int kCols = 8;
         for (int c0 = tid; c0 < L.in; c0 += nthr * kCols) {
-            float v[kCols][BT];
+            float v[kCols];
 #pragma unroll
             for (int u = 0; u < kCols; ++u)
+                if (c0 + u * nthr < L.in) v[u] = x[(size_t)b0 * L.in + c0 + u * nthr];
 #pragma unroll
-                for (int b = 0; b < BT; ++b)
-                    v[u][b] = (b < nb && c0 + u * nthr < L.in) ? to_f32(x[(size_t)(b0 + b) * L.in + c0 + u * nthr]) : 0.0f;
-#pragma unroll
-            for (int u = 0; u < kCols; ++u) {
-                const int c = c0 + u * nthr;
-                if (c < L.in) {
-                    if constexpr (BT == 1) {
-                        xs[c] = v[u][0];
-                    } else if constexpr (BT == 2) {
-                        *reinterpret_cast<float2*>(xs + (size_t)c * 2) = make_float2(v[u][0], v[u][1]);
-                    } else {
-#pragma unroll
-                        for (int q = 0; q < BT / 4; ++q)
-                            *reinterpret_cast<float4*>(xs + (size_t)c * BT + 4 * q) =
-                                make_float4(v[u][4 * q], v[u][4 * q + 1], v[u][4 * q + 2], v[u][4 * q + 3]);
-                    }
-                }
-            }
+            for (int u = 0; u < kCols; ++u)
+                if (c0 + u * nthr < L.in) xs[c0 + u * nthr] = v[u];
         }
     }
-    if (tid < BT) xs[(size_t)L.in * BT + tid] = 0.0f;
+    if (tid == 0) xs[L.in] = 0.0f;
     __syncthreads();
 
     for (int i = 0;;) {
-        float acc[BT];
-#pragma unroll
-        for (int b = 0; b < BT; ++b) acc[b] = 0.0f;
+        float acc = 0.0f;
         if (r >= 0) {
             const size_t row_off = (size_t)r * L.kp;
             for (int v0 = lg;;) {
 #pragma unroll
                 for (int u = 0; u < U; ++u)
 #pragma unroll
-                    for (int e = 0; e < CK::VEC; ++e) gather_fma<BT>(acc, xs, ck[u].col(e), ck[u].weight(e));
+                    for (int e = 0; e < CK::VEC; ++e) acc = fmaf(ck[u].weight(e), xs[ck[u].col(e)], acc);
                 v0 += G * U;
                 if (v0 >= nvec) break;
 #pragma unroll
@@ -391,17 +349,8 @@ __global__ void __launch_bounds__(512) cfi_splitk_kernel(DevLayer L, const VT* _
         }
         // Finish the k-sum across the G lanes of the group.
 #pragma unroll
-        for (int b = 0; b < BT; ++b) {
-            float v = acc[b];
-#pragma unroll
-            for (int m = G >> 1; m > 0; m >>= 1) v += __shfl_xor_sync(0xffffffffu, v, m);
-            acc[b] = v;
-        }
-        if (lg == 0 && o_done < L.out) {
-#pragma unroll
-            for (int b = 0; b < BT; ++b)
-                if (b < nb) from_f32(&y[(size_t)(b0 + b) * L.out + o_done], activate(acc[b] + bias_done, L.act));
-        }
+        for (int m = G >> 1; m > 0; m >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, m);
+        if (lg == 0 && o_done < L.out) y[(size_t)b0 * L.out + o_done] = activate(acc + bias_done, L.act);
         if (!more) break;
     }
 }
@@ -689,6 +638,7 @@ cfi_batch_kernel(DevLayer L, const VT* __restrict__ x, VT* __restrict__ y, int b
     }
 }
 
+#include "cfi_splitk_rows.cuh"
 #include "cfi_dense_tc.cuh"
 #include "cfi_slab.cuh"
 #include "cfi_dense_split.cuh"
@@ -716,31 +666,51 @@ int splitk_lanes_per_row(int nvec, int units) {
     return g;
 }
 
+// fp32 at batch 1 stages x with plain 16-byte loads (cfi_splitk_kernel), everything else row by row (cfi_splitk_rows_kernel).
+bool splitk_by_rows(const cfi_layer* l, int bt) { return l->dtype == CFI_BF16 || bt > 1; }
+
 SplitkShape splitk_shape(const cfi_layer* l, int batch) {
     SplitkShape s{};
-    s.bt = batch >= 8 ? 8 : batch >= 3 ? 4 : batch == 2 ? 2 : 1;
-    while (s.bt > 1 && (size_t)(l->d.in + 1) * s.bt * 4 > (size_t)l->smem_optin) s.bt >>= 1;
+    const int es = l->dtype == CFI_BF16 ? 2 : 4;
+    auto smem_of = [&](int bt) {
+        return splitk_by_rows(l, bt) ? (size_t)splitk_rows_pitch(l->d.in, es) * bt * es : (size_t)(l->d.in + 1) * bt * 4;
+    };
+    s.bt = batch >= 5 ? 8 : batch >= 3 ? 4 : batch == 2 ? 2 : 1;
+    while (s.bt > 1 && smem_of(s.bt) > (size_t)l->smem_optin) s.bt >>= 1;
     const int nvec = l->d.kp / vec_of(l->dtype, l->d.idx16 != 0);
-    s.g = splitk_lanes_per_row(nvec, splitk_units_in_flight(l->dtype == CFI_F32, l->d.idx16 != 0));
+    s.g = splitk_lanes_per_row(nvec, splitk_by_rows(l, s.bt) ? splitk_rows_units(l->dtype == CFI_F32, l->d.idx16 != 0, s.bt)
+                                                             : splitk_units_in_flight(l->dtype == CFI_F32, l->d.idx16 != 0));
     // Every CTA stages x for itself (from L2), so larger CTAs spend less of the L2 bandwidth on x.  The staged x
     // also limits how many CTAs fit an SM; the grid is sized to one wave of what fits (at most eight CTAs per
     // SM), with several rows per group when needed (rows of a group run one after the other).
-    s.smem = (size_t)(l->d.in + 1) * s.bt * 4;
+    s.smem = smem_of(s.bt);
+    s.grid_y = (batch + s.bt - 1) / s.bt;
     const int fit = (int)std::max<size_t>(1, std::min<size_t>(8, ((size_t)227 * 1024) / (s.smem + 1024)));
     const int64_t lanes = (int64_t)l->d.out * s.g;
+    if (splitk_by_rows(l, s.bt)) {
+        // As few CTAs per SM as give every lane a row (at most 512 lanes each, what fits beside the staged x), the rows
+        // spread evenly over them: 5.2 rows of 768 on each of 148 SMs rather than 16 rows on 48.
+        const int64_t lanes_per_sm = (lanes * s.grid_y + l->sm_count - 1) / l->sm_count;
+        const int per_sm = (int)std::max<int64_t>(1, std::min<int64_t>({fit, 4, (lanes_per_sm + 511) / 512}));
+        const int slots = std::max(1, l->sm_count * per_sm / s.grid_y);
+        const int rows = (l->d.out + slots - 1) / slots, at_once = 512 / s.g, warp_rows = 32 / s.g;
+        s.rows_per_group = (rows + at_once - 1) / at_once;
+        int groups = (rows + s.rows_per_group - 1) / s.rows_per_group;
+        groups = std::max((groups + warp_rows - 1) / warp_rows * warp_rows, 128 / s.g);
+        s.threads = groups * s.g;
+        s.grid_x = (l->d.out + groups * s.rows_per_group - 1) / (groups * s.rows_per_group);
+        return s;
+    }
     s.threads = lanes >= (int64_t)l->sm_count * 256 ? 256 : 128;
     if (fit <= 2 && lanes >= (int64_t)l->sm_count * 512) s.threads = 512;
     const int groups = s.threads / s.g;
     const int ctas_one_row_each = (l->d.out + groups - 1) / groups;
-    s.grid_y = (batch + s.bt - 1) / s.bt;
-    const int target = std::max(1, l->sm_count * fit / s.grid_y);  // the batch tiles share the wave
+    const int target = std::max(1, l->sm_count * fit / s.grid_y);  // the batch rows share the wave
     s.rows_per_group = std::max(1, (ctas_one_row_each + target - 1) / target);
     // x loads in flight per staging thread: 8 when 4 would need more than one round and the grid is small enough
     // that the extra registers do not cost a wave.
     s.xs = (l->d.in > 16 * s.threads && s.threads == 128) ? 8 : 4;
     s.grid_x = (l->d.out + groups * s.rows_per_group - 1) / (groups * s.rows_per_group);
-    s.grid_y = (batch + s.bt - 1) / s.bt;
-    s.smem = (size_t)(l->d.in + 1) * s.bt * 4;
     return s;
 }
 
@@ -835,14 +805,18 @@ cfi_status_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, int threads, size_t
 template <typename VT, bool I16, int BT, int G>
 cfi_status_t launch_splitk_g(const cfi_layer* l, const SplitkShape& s, const VT* x, VT* y, int batch,
                              cudaStream_t st) {
-    if (s.xs == 8) {
-        if (cfi_status_t e = set_smem<cfi_splitk_kernel<VT, I16, BT, G, 8>>(s.smem, l->device)) return e;
-        return launch_pdl(cfi_splitk_kernel<VT, I16, BT, G, 8>, dim3(s.grid_x, s.grid_y), s.threads, s.smem, st, l->d, x, y, batch,
+    if constexpr (BT > 1 || sizeof(VT) == 2) {
+        if (cfi_status_t e = set_smem<cfi_splitk_rows_kernel<VT, I16, BT, G>>(s.smem, l->device)) return e;
+        return launch_pdl(cfi_splitk_rows_kernel<VT, I16, BT, G>, dim3(s.grid_x, s.grid_y), s.threads, s.smem, st, l->d, x, y, batch,
                           s.rows_per_group);
+    } else {
+        if (s.xs == 8) {
+            if (cfi_status_t e = set_smem<cfi_splitk_kernel<I16, G, 8>>(s.smem, l->device)) return e;
+            return launch_pdl(cfi_splitk_kernel<I16, G, 8>, dim3(s.grid_x, s.grid_y), s.threads, s.smem, st, l->d, x, y, s.rows_per_group);
+        }
+        if (cfi_status_t e = set_smem<cfi_splitk_kernel<I16, G, 4>>(s.smem, l->device)) return e;
+        return launch_pdl(cfi_splitk_kernel<I16, G, 4>, dim3(s.grid_x, s.grid_y), s.threads, s.smem, st, l->d, x, y, s.rows_per_group);
     }
-    if (cfi_status_t e = set_smem<cfi_splitk_kernel<VT, I16, BT, G, 4>>(s.smem, l->device)) return e;
-    return launch_pdl(cfi_splitk_kernel<VT, I16, BT, G, 4>, dim3(s.grid_x, s.grid_y), s.threads, s.smem, st, l->d, x, y, batch,
-                      s.rows_per_group);
 }
 
 template <typename VT, bool I16, int BT>
@@ -1256,10 +1230,7 @@ cfi_status_t launch_slab(const cfi_layer* l, const void* x, void* y, int batch, 
     return CFI_OK;
 }
 
-// Rate of the gather kernel's arithmetic, used to choose between it and the split-TF32 dense kernel (measured).
-constexpr double kGatherTflops = 12.5;
-
-// The split-k kernel keeps at least one whole row of x (+ one zero element) in shared memory.
+// The split-k kernels keep at least one whole row of x (+ one zero element) in shared memory.
 bool splitk_fits(const cfi_layer* l, int batch) {
     return (l->layouts & CFI_LAYOUT_SMALL_BATCH) && splitk_shape(l, batch).smem <= (size_t)l->smem_optin;
 }
@@ -1278,58 +1249,56 @@ double slab_seconds(const cfi_layer* l, int batch) {
     return 10.8e-6 + 4.4e-12 * (double)l->d.n_active * l->d.k * ((batch + kSlabBT - 1) / kSlabBT);
 }
 
+// Time model of the split-k kernels on batches above one row (measured, chains of launches over 256 .. 4096 features, 80 .. 99 %
+// sparsity, 1 .. 256 rows; within 25 % of the measured times): a launch, the staging of one tile of x, and for every batch
+// tile a part per row (by the lanes that share it) and a part per entry, which costs more in bf16 (two columns to a bank).
+double splitk_seconds(const cfi_layer* l, int batch) {
+    const SplitkShape s = splitk_shape(l, batch);
+    const double eighths = s.bt / 8.0, per_entry = l->dtype == CFI_BF16 ? 3.5e-12 : 2.1e-12;
+    return 2.9e-6 + 14e-9 * (s.smem / 1024.0) + s.grid_y * (0.3e-9 * l->d.out * s.g / 32.0 + per_entry * eighths * l->d.n_active * l->d.k);
+}
+
+// Time model of the tensor-core variant, from the models that choose its launch shape.
+double dense_seconds(const cfi_layer* l, int batch) {
+    if (l->dtype == CFI_F32) {
+        const SplitShape s = split_shape(l, batch);
+        if (!s.ok) return 1e30;
+        return s.seconds - (s.bt <= 64 ? 1.3e-6 : 0.0);  // narrow tiles fill and drain faster than the shapes' common constant says
+    }
+    double t = 0.0;
+    tc_bf16_split(l, batch, &t);
+    return std::max(t, 2.0 * l->out_pad * (double)l->d.in / kSplitHbmBytesPerSecond + 4.7e-6);
+}
+
+// Time model of the gather kernel (measured): the walk over the slabs of x by however many rows a CTA has, and the
+// arithmetic at the rate the gathers sustain; with many batch tiles the re-staging of x by every row tile.
+double gather_seconds(const cfi_layer* l, int batch) {
+    const BatchShape bs = batch_shape(l, batch);
+    if (!bs.ok) return 1e30;
+    const double t_fma = 2.0 * batch * (double)l->d.n_active * l->d.k / 12.5e12;
+    const double t_stage = (double)bs.grid_y * kBatchTile * l->d.in * 4.0 * bs.grid_x / 3.7e12;
+    return std::max(2e-6 + 7e-9 * l->d.in + t_fma, t_fma + t_stage - 0.5 * std::min(t_fma, t_stage) + 5e-6);
+}
+
+// Up to eight rows: split-k.  Above, the fastest by the models among the kernels whose layout the layer holds.  Measured, us a
+// call (split-k / slab / gather / tensor cores): 4096 x 4096 fp32 at 95 %, batch 16 9.4 / 14.1 / 37 / 14.4, batch 64
+// 27 / 41 / 35 / 18; at 99 %, batch 64 11.6 / 30 / 29 / 17.6, batch 256 38 / - / 45 / 40; 768 -> 3072 at 90 %, batch 16
+// 7.6 / 6.1 / 9.4 / 5.9.  bf16 at 99 %: batch 32 7.8 / - / 28 / 13, batch 128 26 / - / 26 / 14.6; at 95 %, batch 32 26 / - / 35 / 13.
 int choose_variant(const cfi_layer* l, int batch) {
     // A layer built without the small-batch layout runs every batch size on what it has.
     if (!(l->layouts & CFI_LAYOUT_SMALL_BATCH) && batch <= 24)
         return l->tc_ok && (batch > 4 || !batch_shape(l, batch).ok) ? CFI_VARIANT_DENSE_TC : fallback_variant(l, batch);
-    // Up to three batch tiles of 8 the split-k kernel (weights re-read from L2 per tile) beats the 64-wide tiles of
-    // the batch kernel, which would be mostly empty.
-    if (batch <= 24) {
-        // Two or three passes of the split-k kernel over a large fp32 layer can take longer than the tensor-core
-        // variant does for any batch up to 128 (measured 4096 x 4096 at 80 %, batch 16: 31 against 25 us; 3072 -> 768:
-        // 22 against 11 us).  A pass of eight batch rows costs about 2.3 us plus the larger of staging x (90 ns per KB
-        // of the 8-row tile, every CTA stages all of it) and the weights (176 G entries per second).
-        if (batch > 8) {
-            constexpr double kNever = 1e30;
-            const double t_stage = (double)l->d.in * 8 * 4 / 1024.0 * 90e-9, t_fma = (double)l->d.n_active * l->d.k / 176e9;
-            const double t_splitk = splitk_fits(l, batch) ? ((batch + 7) / 8) * (2.3e-6 + std::max(t_stage, t_fma)) : kNever;
-            double t_dense = kNever;
-            if (l->tc_ok && l->dtype == CFI_F32) t_dense = split_shape(l, batch).seconds;
-            else if (l->tc_ok) tc_bf16_split(l, batch, &t_dense);
-            // Very sparse fp32 layers: the condensed arrays are far smaller than the dense copy, and the slab kernel
-            // reads only them.
-            if (l->dtype == CFI_F32 && slab_seconds(l, batch) < std::min(t_dense, t_splitk) && slab_shape(l, batch).ok)
-                return CFI_VARIANT_SLAB;
-            if (t_dense < t_splitk) return CFI_VARIANT_DENSE_TC;
-        }
-        return splitk_fits(l, batch) ? CFI_VARIANT_SPLITK : fallback_variant(l, batch);
-    }
-    // bf16 above 24 rows: the dense contraction on the tensor cores beats the gather kernel even at 99 % sparsity
-    // (10 TFLOP/s effective for the gather against several hundred dense), also with a partly empty 128-row tile
-    // now that K can be split over a cluster (3072 -> 768 at batch 64: 8.5 against 33 us).
-    if (l->tc_ok && l->dtype == CFI_BF16) return CFI_VARIANT_DENSE_TC;
-    if (l->tc_ok && l->dtype == CFI_F32) {
-        // fp32: the split-TF32 kernel takes a fixed time per 32-column block of K and tile (it is bound by the
-        // number of MMA instructions), whatever the fill of its 128-row batch tile, and can split K over a cluster
-        // when the tiles are few; the gather kernel's time is its FMAs at the rate it sustains plus the re-staging
-        // of x by every row tile.  Constants fitted to measurements.
-        const BatchShape bs = batch_shape(l, batch);
-        if (!bs.ok) return CFI_VARIANT_DENSE_TC;
-        const double t_dense = split_shape(l, batch).seconds;
-        const double staging = (double)bs.grid_y * kBatchTile * l->d.in * 4.0 * bs.grid_x;
-        // Arithmetic and the re-staging of x overlap about half of the shorter of the two.
-        const double t_fma = 2.0 * batch * (double)l->d.n_active * l->d.k / (kGatherTflops * 1e12), t_stage = staging / 3.7e12;
-        const double t_gather = t_fma + t_stage - 0.5 * std::min(t_fma, t_stage) + 5e-6;
-        if (batch <= 64 && slab_seconds(l, batch) < std::min(t_dense, t_gather) && slab_shape(l, batch).ok) return CFI_VARIANT_SLAB;
-        if (t_dense < t_gather) return CFI_VARIANT_DENSE_TC;
-    }
-    if (batch <= 64 && l->dtype == CFI_F32 && !l->tc_ok && slab_shape(l, batch).ok) {
-        // Without a dense copy: the slab kernel against the gather kernel's 64-wide, partly empty batch tiles.
-        const BatchShape bs = batch_shape(l, batch);
-        if (!bs.ok || slab_seconds(l, batch) < 2.0 * batch * (double)l->d.n_active * l->d.k / (kGatherTflops * 1e12) * (64.0 / std::min(batch, 64)) + 8e-6)
-            return CFI_VARIANT_SLAB;
-    }
-    return fallback_variant(l, batch);
+    if (batch <= 8) return splitk_fits(l, batch) ? CFI_VARIANT_SPLITK : fallback_variant(l, batch);
+    int best = -1;
+    double best_t = 0.0;
+    auto consider = [&](int variant, double t) {
+        if (t < 1e29 && (best < 0 || t < best_t)) best = variant, best_t = t;
+    };
+    if (l->tc_ok) consider(CFI_VARIANT_DENSE_TC, dense_seconds(l, batch));
+    if (batch <= 256 && splitk_fits(l, batch)) consider(CFI_VARIANT_SPLITK, splitk_seconds(l, batch));
+    if (batch <= 64 && l->dtype == CFI_F32 && slab_shape(l, batch).ok) consider(CFI_VARIANT_SLAB, slab_seconds(l, batch));
+    if (!(l->tc_ok && l->dtype == CFI_BF16)) consider(CFI_VARIANT_BATCH, gather_seconds(l, batch));  // bf16 tensor cores always beat it
+    return best >= 0 ? best : fallback_variant(l, batch);
 }
 
 // ------------------------------------------------------------------------------------------------
