@@ -190,6 +190,16 @@ cfi_status_t cfi_pack_device(const float* w_dense, const uint8_t* mask, int32_t 
                              int32_t* indices, int32_t* active_rows, cfi_stream_t stream);
 
 /*
+ * cfi_pack_device_fill — the arrays of a layer whose size query (cfi_pack_device with NULL arrays) has just been made with
+ * the same mask and workspace, both untouched since: the rows are not counted again.  k and n_active are what the query
+ * returned, both at least 1; where the workspace holds other counts nothing is written.  Waits for `stream`.  Errors as
+ * cfi_pack_device.
+ */
+cfi_status_t cfi_pack_device_fill(const float* w_dense, const uint8_t* mask, int32_t out_features, int32_t in_features,
+                                  void* workspace, size_t workspace_bytes, int32_t k, int32_t n_active, float* values,
+                                  int32_t* indices, int32_t* active_rows, cfi_stream_t stream);
+
+/*
  * cfi_create — build a device-resident layer from condensed arrays (the inputs w and indx of
  * Algorithm 1, plus the bias that Sec. 4.4 extracts with the weights).
  *

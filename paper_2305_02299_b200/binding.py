@@ -25,7 +25,7 @@ _ACTS = {"none": ACT_NONE, None: ACT_NONE, "gelu": ACT_GELU, ACT_NONE: ACT_NONE,
 _VARIANTS = {"auto": 0, "simple": 1, "splitk": 2, "batch": 3, "dense_tc": 4, "slab": 5, 0: 0, 1: 1, 2: 2, 3: 3, 4: 4, 5: 5}
 
 EXPORTS = ("cfi_status_string", "cfi_pack", "cfi_compact_producer", "cfi_compact_consumer", "cfi_srigl_workspace_bytes",
-           "cfi_srigl_update", "cfi_pack_device", "cfi_create", "cfi_create_layouts", "cfi_layer_add_layouts", "cfi_forward", "cfi_forward_variant", "cfi_forward_dense",
+           "cfi_srigl_update", "cfi_pack_device", "cfi_pack_device_fill", "cfi_create", "cfi_create_layouts", "cfi_layer_add_layouts", "cfi_forward", "cfi_forward_variant", "cfi_forward_dense",
            "cfi_forward_host",
            "cfi_layer_info", "cfi_choose_variant", "cfi_dense_tile_shape", "cfi_device_status", "cfi_destroy",
            "cfi_stack_create", "cfi_stack_forward", "cfi_stack_destroy", "cfi_stack_forward_static",
@@ -77,6 +77,7 @@ def _load() -> ctypes.CDLL:
     lib.cfi_srigl_workspace_bytes.argtypes = [ci, ci, ctypes.POINTER(ctypes.c_size_t)]
     lib.cfi_srigl_update.argtypes = [vp, vp, vp, ci, ci, ctypes.c_int64, ctypes.c_float, vp, ctypes.c_size_t, i32p, i32p, vp]
     lib.cfi_pack_device.argtypes = [vp, vp, ci, ci, vp, ctypes.c_size_t, i32p, i32p, vp, vp, vp, vp]
+    lib.cfi_pack_device_fill.argtypes = [vp, vp, ci, ci, vp, ctypes.c_size_t, ci, ci, vp, vp, vp, vp]
     lib.cfi_create.argtypes = [f32p, i32p, i32p, f32p, ci, ci, ci, ci, ctypes.c_int, ctypes.c_int, ctypes.POINTER(vp)]
     lib.cfi_create_layouts.argtypes = [f32p, i32p, i32p, f32p, ci, ci, ci, ci, ctypes.c_int, ctypes.c_int, ci, ctypes.POINTER(vp)]
     lib.cfi_layer_add_layouts.argtypes = [vp, ci]
@@ -283,8 +284,8 @@ def cfi_pack_device(w, mask, stream=None):
     indices = torch.empty((na.value, k.value), dtype=torch.int32, device=w.device)
     rows = torch.empty((na.value,), dtype=torch.int32, device=w.device)
     if na.value:
-        _check(_lib.cfi_pack_device(_dev_ptr(w), _dev_ptr(mask), out_f, in_f, base, 8 * out_f + 256, ctypes.byref(k),
-                                    ctypes.byref(na), _dev_ptr(values), _dev_ptr(indices), _dev_ptr(rows), st), "cfi_pack_device")
+        _check(_lib.cfi_pack_device_fill(_dev_ptr(w), _dev_ptr(mask), out_f, in_f, base, 8 * out_f + 256, k.value, na.value,
+                                         _dev_ptr(values), _dev_ptr(indices), _dev_ptr(rows), st), "cfi_pack_device_fill")
     return values, indices, rows
 
 

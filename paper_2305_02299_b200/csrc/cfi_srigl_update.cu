@@ -892,19 +892,23 @@ __global__ void __launch_bounds__(kThreads) pack_rows_kernel(const uint8_t* mask
 }
 
 // One warp per row: its kept entries in increasing column order to values / indices of its rank.  A lane takes VEC
-// consecutive columns, their place follows from a prefix count over the warp.
+// consecutive columns, their place follows from a prefix count over the warp.  n_active and k are the sizes of the arrays
+// where they are known before the launch: nothing is written outside them, nor at all where the counts are others.  -1: as counted.
 template <int VEC>
 __global__ void __launch_bounds__(kThreads) pack_fill_kernel(const float* w, const uint8_t* mask, const int* row_rank, int out_f, int in_f,
-                                                             const PackInfo* info, float* values, int32_t* indices, int32_t* active_rows) {
+                                                             const PackInfo* info, int n_active, int k, float* values, int32_t* indices,
+                                                             int32_t* active_rows) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t r = (int64_t)blockIdx.x * (kThreads / 32) + warp;
-    if (!info->constant || r >= out_f) return;
+    if (k < 0) n_active = info->n_active, k = info->k;
+    if (!info->constant || info->n_active != n_active || info->k != k || r >= out_f) return;
     const int rank = row_rank[r];
-    if (rank < 0) return;
+    if (rank < 0 || rank >= n_active) return;
     if (lane == 0) active_rows[rank] = (int32_t)r;
     const float* wr = w + (size_t)r * in_f;
     const uint8_t* mr = mask + (size_t)r * in_f;
-    size_t at0 = (size_t)rank * info->k;
+    const size_t end = (size_t)(rank + 1) * k;
+    size_t at0 = (size_t)rank * k;
     unsigned int next = kept_set<VEC>(mr, lane * VEC, in_f);
     for (int c0 = 0; c0 < in_f; c0 += 32 * VEC) {
         unsigned int bits = next;
@@ -917,7 +921,7 @@ __global__ void __launch_bounds__(kThreads) pack_fill_kernel(const float* w, con
             if (lane >= off) incl += up;
         }
         size_t at = at0 + (incl - mine);
-        while (bits) {
+        while (bits && at < end) {
             const int c = col + __ffs(bits) - 1;
             bits &= bits - 1;
             values[at] = wr[c];
@@ -1009,39 +1013,74 @@ extern "C" cfi_status_t cfi_srigl_update(float* w, uint8_t* mask, const float* g
     return CFI_OK;
 }
 
+namespace {
+
+struct PackWorkspace {
+    int *row_count, *row_rank;
+    PackInfo* info;
+};
+cfi_status_t pack_workspace(const void* w, const uint8_t* mask, void* workspace, size_t bytes, int32_t out_f, int32_t in_f, PackWorkspace* out) {
+    if (!w || !mask || !workspace) return CFI_ERR_NULL;
+    if (out_f < 1 || in_f < 1 || (int64_t)out_f * in_f > ((int64_t)1 << 31)) return CFI_ERR_SHAPE;
+    if (((uintptr_t)workspace & 255) != 0) return CFI_ERR_ALIGNMENT;
+    if (bytes < (size_t)out_f * 8 + 256) return CFI_ERR_BUFFER_TOO_SMALL;
+    out->row_count = static_cast<int*>(workspace);
+    out->row_rank = out->row_count + out_f;
+    out->info = reinterpret_cast<PackInfo*>(out->row_rank + out_f);
+    return CFI_OK;
+}
+bool pack_vector_loads(const uint8_t* mask, int32_t in_f) { return (in_f & 15) == 0 && ((uintptr_t)mask & 15) == 0; }
+int pack_blocks(int32_t out_f) { return (int)(((int64_t)out_f + kThreads / 32 - 1) / (kThreads / 32)); }
+
+cfi_status_t pack_fill(const PackWorkspace& ws, const float* w, const uint8_t* mask, int32_t out_f, int32_t in_f, int32_t k, int32_t n_active,
+                       float* values, int32_t* indices, int32_t* active_rows, cudaStream_t st) {
+    const auto kernel = pack_vector_loads(mask, in_f) ? pack_fill_kernel<16> : pack_fill_kernel<1>;
+    kernel<<<pack_blocks(out_f), kThreads, 0, st>>>(w, mask, ws.row_rank, out_f, in_f, ws.info, n_active, k, values, indices, active_rows);
+    return cudaGetLastError() == cudaSuccess ? CFI_OK : CFI_ERR_CUDA;
+}
+
+}  // namespace
+
 extern "C" cfi_status_t cfi_pack_device(const float* w_dense, const uint8_t* mask, int32_t out_features, int32_t in_features,
                                         void* workspace, size_t workspace_bytes, int32_t* k, int32_t* n_active, float* values,
                                         int32_t* indices, int32_t* active_rows, cfi_stream_t stream) {
-    if (!w_dense || !mask || !workspace || !k || !n_active) return CFI_ERR_NULL;
-    if (out_features < 1 || in_features < 1 || (int64_t)out_features * in_features > ((int64_t)1 << 31)) return CFI_ERR_SHAPE;
+    if (!k || !n_active) return CFI_ERR_NULL;
     const bool fill = values || indices || active_rows;
     if (fill && !(values && indices && active_rows)) return CFI_ERR_NULL;
-    if (((uintptr_t)workspace & 255) != 0) return CFI_ERR_ALIGNMENT;
-    if (workspace_bytes < (size_t)out_features * 8 + 256) return CFI_ERR_BUFFER_TOO_SMALL;
-    int* row_count = static_cast<int*>(workspace);
-    int* row_rank = row_count + out_features;
-    PackInfo* info = reinterpret_cast<PackInfo*>(row_rank + out_features);
+    PackWorkspace ws;
+    if (cfi_status_t e = pack_workspace(w_dense, mask, workspace, workspace_bytes, out_features, in_features, &ws)) return e;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    const bool vec = (in_features & 15) == 0 && ((uintptr_t)mask & 15) == 0;
-    const int blocks = (int)(((int64_t)out_features + kThreads / 32 - 1) / (kThreads / 32));
     PackInfo host{};
-    if (cudaMemsetAsync(info, 0, sizeof(PackInfo), st) != cudaSuccess) {
-        cudaGetLastError();
-        return CFI_ERR_CUDA;
+    bool ok = cudaMemsetAsync(ws.info, 0, sizeof(PackInfo), st) == cudaSuccess;
+    if (ok) {
+        const auto kernel = pack_vector_loads(mask, in_features) ? pack_rows_kernel<16> : pack_rows_kernel<1>;
+        kernel<<<pack_blocks(out_features), kThreads, 0, st>>>(mask, out_features, in_features, ws.row_count, ws.row_rank, ws.info);
+        ok = cudaGetLastError() == cudaSuccess;
     }
-    if (vec) pack_rows_kernel<16><<<blocks, kThreads, 0, st>>>(mask, out_features, in_features, row_count, row_rank, info);
-    else pack_rows_kernel<1><<<blocks, kThreads, 0, st>>>(mask, out_features, in_features, row_count, row_rank, info);
-    if (fill) {  // writes nothing where the fan-in is not constant
-        if (vec) pack_fill_kernel<16><<<blocks, kThreads, 0, st>>>(w_dense, mask, row_rank, out_features, in_features, info, values, indices, active_rows);
-        else pack_fill_kernel<1><<<blocks, kThreads, 0, st>>>(w_dense, mask, row_rank, out_features, in_features, info, values, indices, active_rows);
-    }
-    if (cudaGetLastError() != cudaSuccess || cudaMemcpyAsync(&host, info, sizeof(host), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaStreamSynchronize(st) != cudaSuccess) {
+    if (ok && fill) ok = pack_fill(ws, w_dense, mask, out_features, in_features, -1, -1, values, indices, active_rows, st) == CFI_OK;
+    ok = ok && cudaMemcpyAsync(&host, ws.info, sizeof(host), cudaMemcpyDeviceToHost, st) == cudaSuccess && cudaStreamSynchronize(st) == cudaSuccess;
+    if (!ok) {
         cudaGetLastError();
         return CFI_ERR_CUDA;
     }
     if (!host.constant) return CFI_ERR_NOT_CONSTANT_FAN_IN;
     *n_active = host.n_active;
     *k = host.n_active ? host.k : 0;
+    return CFI_OK;
+}
+
+extern "C" cfi_status_t cfi_pack_device_fill(const float* w_dense, const uint8_t* mask, int32_t out_features, int32_t in_features,
+                                             void* workspace, size_t workspace_bytes, int32_t k, int32_t n_active, float* values,
+                                             int32_t* indices, int32_t* active_rows, cfi_stream_t stream) {
+    if (!values || !indices || !active_rows) return CFI_ERR_NULL;
+    if (k < 1 || n_active < 1 || n_active > out_features || k > in_features) return CFI_ERR_SHAPE;
+    PackWorkspace ws;
+    if (cfi_status_t e = pack_workspace(w_dense, mask, workspace, workspace_bytes, out_features, in_features, &ws)) return e;
+    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+    if (pack_fill(ws, w_dense, mask, out_features, in_features, k, n_active, values, indices, active_rows, st) != CFI_OK ||
+        cudaStreamSynchronize(st) != cudaSuccess) {
+        cudaGetLastError();
+        return CFI_ERR_CUDA;
+    }
     return CFI_OK;
 }

@@ -213,3 +213,30 @@ def test_pack_device_errors_and_empty():
     assert e.value.status == 3
     v, ix, rows = cfi.cfi_pack_device(torch.zeros((4, 8), device="cuda"), torch.zeros((4, 8), device="cuda", dtype=torch.uint8))
     assert v.shape == (0, 0) and rows.shape == (0,)
+
+
+def test_pack_device_fill_writes_only_what_was_counted():
+    """The filling step takes the counts of the size query; with other counts it writes nothing."""
+    import ctypes
+    import torch
+    from paper_2305_02299_b200 import binding as cfi
+    out_f, in_f, k = 40, 96, 7
+    L = inputs.make_layer(in_f, out_f, k, n_ablated=3, seed=5)
+    w, m = torch.from_numpy(L.w_dense).cuda(), torch.from_numpy(L.mask).cuda()
+    ws = torch.empty(8 * out_f + 512, dtype=torch.uint8, device="cuda")
+    base = (ws.data_ptr() + 255) & ~255
+    kk, na = ctypes.c_int32(0), ctypes.c_int32(0)
+    head = (w.data_ptr(), m.data_ptr(), out_f, in_f, base, 8 * out_f + 256)
+    assert cfi._lib.cfi_pack_device(*head, ctypes.byref(kk), ctypes.byref(na), None, None, None, None) == 0
+    assert (kk.value, na.value) == (k, out_f - 3)
+    v = torch.full((out_f, in_f), -1.0, device="cuda")
+    ix, rows = torch.full((out_f, in_f), -1, dtype=torch.int32, device="cuda"), torch.full((out_f,), -1, dtype=torch.int32, device="cuda")
+    arrays = (v.data_ptr(), ix.data_ptr(), rows.data_ptr(), None)
+    for wrong in ((k - 1, out_f - 3), (k, out_f - 4), (k + 1, out_f - 3)):
+        assert cfi._lib.cfi_pack_device_fill(*head, *wrong, *arrays) == 0
+        assert bool((v == -1).all()) and bool((ix == -1).all()) and bool((rows == -1).all())
+    assert cfi._lib.cfi_pack_device_fill(*head, k, out_f - 3, *arrays) == 0
+    hv, hix, hrows = cfi.cfi_pack(L.w_dense, L.mask)
+    n = hv.size
+    assert np.array_equal(v.flatten()[:n].cpu().numpy(), hv.ravel()) and np.array_equal(ix.flatten()[:n].cpu().numpy(), hix.ravel())
+    assert np.array_equal(rows[:out_f - 3].cpu().numpy(), hrows) and bool((v.flatten()[n:] == -1).all())
