@@ -13,7 +13,7 @@
 // the lists.  Per neuron one 11-bit digit leaves a few dozen open, which are ranked against one another.  A layer with
 // so many equal keys that the open elements do not fit the lists takes further digits first, at last of the position.
 //
-// 4096 x 4096 at 80 %, K = 30 % of the weights, four kernels: 34 + 41 + 16 + 73 us, 0.20 ms with the host's wait
+// 4096 x 4096 at 80 %, K = 30 % of the weights, four kernels: 34 + 41 + 16 + 60 us, 0.19 ms with the host's wait
 // (before: four sweeps of 8-bit digits, flags for every entry and a four-digit selection per neuron, 12 kernels: 0.39 ms);
 // 3072 x 768 at 90 %: 17 + 19 + 13 + 19 us, 0.10 ms (0.17 ms).  Moved per entry: 9 bytes in each of the two sweeps and the
 // per-neuron step, and what changes: 30 against 50.
@@ -486,17 +486,44 @@ struct SelectSmem {
     unsigned int part[T / 32], n;
     Pick pick;
 };
+//
+// Where the caller knows the smallest key (base, else 0), the first histogram is of 64 bins a binade from there on instead of
+// the 11 leading bits, which are 8 a binade: most gradients of a row lie within two binades of one another, so with those a
+// warp's counts met in a few bins and were added one after the other (4096 x 4096: finalize_kernel 73 -> 60 us).  A bin that holds too many all the same (its elements equal, or 32 binades and more away) leaves it to the leading bits.
+constexpr int kFineShift = 23 - 6;
 template <int T, typename Visit>
-__device__ unsigned long long block_select(unsigned int want, unsigned int count, Visit visit, SelectSmem<T>& sm) {
+__device__ unsigned long long block_select(unsigned int want, unsigned int count, Visit visit, SelectSmem<T>& sm, unsigned int base = 0) {
     const int t = threadIdx.x;
-    unsigned long long prefix = 0;
-    int shift = kAllBits;
-    while (count > T && shift > 0) {
-        const int digit = shift < 11 ? shift : 11;
-        constexpr int kPer = kRowBins / T;
+    constexpr int kPer = kRowBins / T;
+    auto clear = [&]() {
 #pragma unroll
         for (int i = 0; i < kPer / 4; ++i) reinterpret_cast<uint4*>(sm.hist)[i * T + t] = make_uint4(0u, 0u, 0u, 0u);
         __syncthreads();
+    };
+    auto find = [&]() {
+        __syncthreads();
+        unsigned int bins[kPer];
+#pragma unroll
+        for (int i = 0; i < kPer / 4; ++i) {
+            const uint4 q = reinterpret_cast<const uint4*>(sm.hist)[t * (kPer / 4) + i];
+            bins[4 * i] = q.x, bins[4 * i + 1] = q.y, bins[4 * i + 2] = q.z, bins[4 * i + 3] = q.w;
+        }
+        return block_pick<T>(want, bins, sm.part, sm.pick);
+    };
+    unsigned long long prefix = 0;
+    int shift = kAllBits;
+    bool fine = false;
+    unsigned int fine_bin = 0;
+    if (base != 0 && count > T) {
+        clear();
+        visit([&](unsigned int key, unsigned int) { atomicAdd(&sm.hist[min((key - base) >> kFineShift, kRowBins - 1u)], 1u); });
+        const Pick p = find();
+        if (p.count <= T) fine = true, fine_bin = p.bin, want -= p.below, count = p.count;
+        __syncthreads();
+    }
+    while (!fine && count > T && shift > 0) {
+        const int digit = shift < 11 ? shift : 11;
+        clear();
         if (shift == kAllBits) {
             visit([&](unsigned int key, unsigned int) { atomicAdd(&sm.hist[key >> (kKeyBits - 11)], 1u); });
         } else {
@@ -505,14 +532,7 @@ __device__ unsigned long long block_select(unsigned int want, unsigned int count
                     atomicAdd(&sm.hist[composite_top(key, pos, shift - digit) & ((1u << digit) - 1u)], 1u);
             });
         }
-        __syncthreads();
-        unsigned int bins[kPer];
-#pragma unroll
-        for (int i = 0; i < kPer / 4; ++i) {
-            const uint4 q = reinterpret_cast<const uint4*>(sm.hist)[t * (kPer / 4) + i];
-            bins[4 * i] = q.x, bins[4 * i + 1] = q.y, bins[4 * i + 2] = q.z, bins[4 * i + 3] = q.w;
-        }
-        const Pick p = block_pick<T>(want, bins, sm.part, sm.pick);
+        const Pick p = find();
         want -= p.below, count = p.count;
         prefix = (prefix << digit) | p.bin;
         shift -= digit;
@@ -523,7 +543,11 @@ __device__ unsigned long long block_select(unsigned int want, unsigned int count
         const unsigned int at = atomicAdd(&sm.n, 1u);
         if (at < T) sm.open[at] = composite(key, pos);
     };
-    if (shift >= kPosBits) {  // the usual end: a key digit left few enough
+    if (fine) {  // the usual end
+        visit([&](unsigned int key, unsigned int pos) {
+            if (min((key - base) >> kFineShift, kRowBins - 1u) == fine_bin) list(key, pos);
+        });
+    } else if (shift >= kPosBits) {  // a key digit left few enough
         const int key_shift = shift - kPosBits;
         const unsigned int top = (unsigned int)prefix;
         visit([&](unsigned int key, unsigned int pos) {
@@ -633,8 +657,8 @@ __global__ void __launch_bounds__(kThreads) resolve_kernel(const uint2* list, un
 // 9 bytes read per entry, and of the outputs only what changes is written (a masked-off weight is 0 already, a kept one
 // keeps its value); bound by instruction issue as much as by memory, hence the one key per column: columns that cannot be
 // chosen carry kNoKey, above every key, and every later step is a compare (4096 x 4096: 105 us with 62-bit compares per
-// column, 73 with these).  The selection takes two visits of the row as a
-// rule: one 11-bit digit, then the few dozen elements left in its bin are ranked against one another.
+// column, 73 with these, 60 with the finer first histogram of block_select).  The selection takes two visits of the row as a
+// rule: one histogram, then the few elements left in its bin are ranked against one another.
 constexpr unsigned int kNoKey = 0xFFFFFFFFu;
 template <int VEC, int COLS, int T>
 __global__ void __launch_bounds__(T, (COLS > 2048 ? 1024 : 1536) / T) finalize_kernel(float* w, uint8_t* mask, const float* grad, const uint8_t* survives,
@@ -676,7 +700,8 @@ __global__ void __launch_bounds__(T, (COLS > 2048 ? 1024 : 1536) / T) finalize_k
         const bool dropped = u < cut_key || (u == cut_key && (long long)(col + e) <= cut_col);
         return c.on(e) && !(on0 && dropped);
     };
-    unsigned int key[kChunks][VEC], kept_bits[kChunks];
+    __shared__ unsigned int least[T / 32];
+    unsigned int key[kChunks][VEC], kept_bits[kChunks], lowest = kNoKey;
     int mine = 0;
     if (kCached) {
 #pragma unroll
@@ -689,9 +714,12 @@ __global__ void __launch_bounds__(T, (COLS > 2048 ? 1024 : 1536) / T) finalize_k
                 if (!kept && __float_as_uint(c[u].w(e)) != 0u) wr[col + e] = 0.0f;  // pruned, or free (a weight grown later starts at 0)
                 kept_bits[u] |= kept ? 1u << e : 0u;
                 key[u][e] = kept || col >= in_f ? kNoKey : grad_key(c[u].g(e));
+                lowest = min(lowest, key[u][e]);
             }
             mine += __popc(kept_bits[u]);
         }
+        lowest = __reduce_min_sync(0xffffffffu, lowest);
+        if ((t & 31) == 0) least[t >> 5] = lowest;
     } else {
         for (int col = t * VEC; col < in_f; col += T * VEC) {
             Cols<VEC> v;
@@ -702,6 +730,10 @@ __global__ void __launch_bounds__(T, (COLS > 2048 ? 1024 : 1536) / T) finalize_k
         }
     }
     const int kept = block_sum<T>(mine, part, 0);
+    if (kCached) {
+#pragma unroll
+        for (int i = 0; i < T / 32; ++i) lowest = min(lowest, least[i]);
+    }
     const bool trim = kept > k_new;
     const int m = trim ? kept - k_new : k_new - kept;
     if (kCached && trim) {  // the other keys: magnitudes of the kept weights
@@ -731,7 +763,7 @@ __global__ void __launch_bounds__(T, (COLS > 2048 ? 1024 : 1536) / T) finalize_k
                         if (is_kept(v, e, col) == trim) f(trim ? weight_key(v.w(e)) : grad_key(v.g(e)), (unsigned int)(col + e));
                 }
             }
-        }, sm);
+        }, sm, kCached && !trim ? lowest : 0u);
     }
     const unsigned int row_key = (unsigned int)(cut >> kPosBits), row_col = (unsigned int)(cut & 0x7FFFFFFFull);
     auto chosen = [&](unsigned int k, int col) { return m > 0 && (k < row_key || (k == row_key && (unsigned int)col <= row_col)); };

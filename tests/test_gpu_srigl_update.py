@@ -240,3 +240,21 @@ def test_pack_device_fill_writes_only_what_was_counted():
     n = hv.size
     assert np.array_equal(v.flatten()[:n].cpu().numpy(), hv.ravel()) and np.array_equal(ix.flatten()[:n].cpu().numpy(), hix.ravel())
     assert np.array_equal(rows[:out_f - 3].cpu().numpy(), hrows) and bool((v.flatten()[n:] == -1).all())
+
+
+@pytest.mark.parametrize("in_f", [132, 768, 1030, 4096])
+@pytest.mark.parametrize("kind", ["wide", "equal", "inf"])
+def test_regrowth_where_the_fine_histogram_cannot_part_the_gradients(in_f, kind):
+    """Gradients over 60 binades, nearly all equal, and with infinities: the first histogram of a row's selection puts
+    too many into one bin, and the leading bits decide."""
+    rng = np.random.default_rng(in_f)
+    w, m, _ = _layer(24, in_f, max(2, in_f // 12), 2, seed=in_f)
+    g = rng.standard_normal(w.shape).astype(np.float32)
+    if kind == "wide":
+        g = (g * np.exp2(rng.uniform(-60, 0, w.shape))).astype(np.float32)
+        g[:, 0] = 1.0
+    elif kind == "equal":
+        g = np.where(rng.random(w.shape) < 0.97, np.float32(0.25), g).astype(np.float32)
+    else:
+        g[:, 1] = np.inf
+    _compare(w, m, g, int(0.3 * m.sum()), 0.3)
