@@ -22,24 +22,26 @@
 //
 // The layer keeps one dense fp32 copy of its weight, Wd[out_pad][in] (zero rows for ablated and padding rows).  A tile
 // is 128 output rows (M) x BT batch rows (N side), so a small batch costs a narrow MMA and not a mostly empty 128-row
-// tile.  Per 32-column block of K, in a ring of four to eight stages [Wd box | x box | x_lo]:
+// tile.  Per 32-column block of K, in a ring of four or six stages [Wd box | x box | x_lo]:
 //   warp 0, one lane    TMA: the 128 x 32 box of Wd and the BT x 32 box of x (fp32, 128-byte swizzle).  The weight
 //                       boxes of the first ring round are requested before the wait for the kernel ahead;
 //   warps 3..18         two teams of eight worker warps; team t prepares the blocks i = t (mod 2).  x_lo: the x box is
 //                       read back from shared memory, x - (x with the low 13 bits cleared) is written right behind
-//                       it in the same swizzled layout, so that [x; x_lo] reads as one K-major operand of 2 BT rows.
-//                       w_lo: two threads per output row read that row's 128 bytes of the Wd box and write the lo
-//                       parts straight into tensor memory (tcgen05.st), from where the second MMA takes its A
-//                       operand.  tcgen05.wait::st and fence.proxy.async, then one arrival per warp on the stage's
-//                       "ready" barrier;
-//   warps 1 and 2, one lane each   two MMA issuers (kind::tf32, M = 128, K = 8).  Warp 1 issues  Wd x [x; x_lo]
-//                       (A = the Wd box in shared memory, N = 2 BT) into accumulator columns 0 .. 2BT-1, warp 2 issues
-//                       w_lo x x  (A from tensor memory, N = BT) into columns 2BT .. 3BT-1.  One thread gets an MMA
-//                       accepted about every 143 cycles whatever its size (measured on this part), two threads get
-//                       two; separate accumulators keep the two streams independent.  Each issuer's tcgen05.commit
-//                       arrives on the stage's "empty" barrier (count 2), which the TMA lane waits for.
-// After the last block the workers add the three accumulator parts, add the bias, apply the activation and store: a
+//                       it in the same swizzled layout.  The weight: two threads per output row read that row's 128
+//                       bytes of the Wd box and write both of its parts into tensor memory (tcgen05.st), from where
+//                       every MMA takes its A operand.  tcgen05.wait::st and fence.proxy.async, then one arrival per
+//                       warp on the stage's "ready" barrier;
+//   warps 1 and 2, one lane each   two MMA issuers (kind::tf32, M = 128, N = BT, K = 8).  Warp 1 issues w_hi x x into
+//                       accumulator columns 0 .. BT-1, warp 2 w_hi x x_lo and w_lo x x into columns BT .. 2BT-1.
+//                       Each issuer's tcgen05.commit arrives on the stage's "empty" barrier (count 2), which the TMA
+//                       lane waits for.
+// After the last block the workers add the two accumulators, add the bias, apply the activation and store: a
 // tensor-memory lane is an output row, so for one batch row a warp writes 32 consecutive outputs, 128 contiguous bytes.
+//
+// What bounds the main loop is shared-memory traffic beside the tensor pipe: per block 16 KB + 128 BT bytes come in, the
+// workers read as much and write 128 BT bytes, the MMAs read 384 BT.  With w_hi read from the Wd box instead (another 16 KB
+// a block, and three accumulators) a block took 0.345 us at BT = 64 and 0.515 at BT = 128, now 0.26 and 0.46 (tensor pipe
+// alone: 0.21 and 0.42).  3072 -> 768 at batch 1576: 46.5 -> 40.9 us with BT = 96; 4096 x 4096 at batch 64: 16.3 -> 15.1.
 //
 // Split K over a thread-block cluster (cluster dimension z) as in the bf16 kernel: CTA r contracts the r-th share of
 // the K blocks, leaves its partial tile [BT][128] in its shared memory, and after the hardware cluster barrier sums its
@@ -51,16 +53,19 @@
 constexpr int kSpM = 128, kSpK = 32;
 constexpr int kSpTeamWarps = 8, kSpTeams = 2, kSpWorkerWarps = kSpTeams * kSpTeamWarps, kSpFirstWorker = 3;
 constexpr int kSpThreads = 32 * (kSpFirstWorker + kSpWorkerWarps);
-// Batch tiles of the kernel (the MMA's N is BT and 2 BT, multiples of 16 up to 256) and the ring depth each one affords
-// in shared memory (16 KB + 256 BT bytes per stage) and tensor memory (3 BT accumulator columns + 32 per stage).
+// Batch tiles of the kernel (the MMA's N is BT, a multiple of 16) and the ring depth each one affords in shared memory
+// (16 KB + 256 BT bytes per stage) and tensor memory (2 BT accumulator columns + 64 per stage).
 constexpr int kSpTiles[] = {16, 32, 48, 64, 96, 128};
 constexpr int kSpNumTiles = sizeof(kSpTiles) / sizeof(kSpTiles[0]);
+// A launch may use fewer rows of its tiles, in steps of 16 (the MMA's N): 80 of 96, or 112 of 128, where that fills the SMs
+// better or leaves less of the last tile empty.  3072 -> 768 at batch 1576: 20 x 6 tiles of 80 rows 37.4 us, 17 x 6 of 96 40.9.
+constexpr int kSpRowStep = 16;
 // The depth is a multiple of the number of worker teams, so that a ring slot always belongs to the same team: a team
 // that met only every other phase of a slot's barrier could not tell a phase from the one two before it by parity.
-__host__ __device__ constexpr int sp_stages(int bt) { return bt >= 96 ? 4 : bt >= 48 ? 6 : 8; }
+__host__ __device__ constexpr int sp_stages(int bt) { return bt >= 96 ? 4 : 6; }
 constexpr int kMaxClusterSplit = 8;  // largest portable thread-block cluster
 constexpr uint32_t kSpWBytes = kSpM * kSpK * 4;  // one weight box: 16 KB
-constexpr uint32_t kSpTmemCols = 512;            // 3 BT accumulator columns ... one 32-column w_lo stage per ring slot at the top
+constexpr uint32_t kSpTmemCols = 512;            // 2 BT accumulator columns ... one stage of 2 x 32 weight columns per ring slot at the top
 __host__ __device__ constexpr uint32_t sp_x_bytes(int bt) { return (uint32_t)bt * kSpK * 4; }  // the x box; x_lo has the same size
 __host__ __device__ constexpr uint32_t sp_stage_bytes(int bt) { return kSpWBytes + 2 * sp_x_bytes(bt); }
 __host__ __device__ constexpr uint32_t sp_data_bytes(int bt) {  // the ring, or the partial tile of a K split if that is larger
@@ -71,14 +76,6 @@ __host__ __device__ constexpr size_t sp_smem_bytes(int bt) { return 1024 + (size
 // fp32 accumulate, tf32 x tf32, both K-major, M = 128, N = n.
 __host__ __device__ constexpr uint32_t sp_instr_desc(int n) {
     return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(kSpM >> 4) << 24);
-}
-// Both operands from shared memory.
-__device__ __forceinline__ void umma_tf32_ss(uint32_t tmem_d, uint64_t desc_a, uint64_t desc_b, uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, {%5, %5, %5, %5}, p;\n\t}" ::"r"(tmem_d),
-        "l"(desc_a), "l"(desc_b), "r"(idesc), "r"(accumulate), "r"(0u)
-        : "memory");
 }
 // A operand from tensor memory (row m in lane m, 32-bit elements in consecutive columns), B from shared memory.
 __device__ __forceinline__ void umma_tf32_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t desc_b, uint32_t idesc, uint32_t accumulate) {
@@ -104,11 +101,11 @@ __device__ __forceinline__ float tf32_lo(float v) { return v - __uint_as_float(_
 // batch row (4 outputs each), 16 rows per pass, 512-byte runs of y.  The loads of kRows rows (NS each; the CTA's own tile
 // is read as ordinary shared memory) are all issued before the first sum needs one, so that the latency of distributed
 // shared memory is paid once per kRows rows.
-template <int BT, int NS>
-__device__ __forceinline__ void sp_reduce(const DevLayer& L, float* __restrict__ y, int batch, int n0, int b0, uint32_t base, int split,
-                                          int wt) {
+template <int NS>
+__device__ __forceinline__ void sp_reduce(const DevLayer& L, float* __restrict__ y, int batch, int n0, int b0, int rows, uint32_t base,
+                                          int split, int wt) {
     constexpr int kRows = NS <= 2 ? 4 : NS <= 4 ? 2 : 1;
-    const int ch = wt & 31, rows_per = (BT + NS - 1) / NS, o = n0 + 4 * ch;
+    const int ch = wt & 31, rows_per = (rows + NS - 1) / NS, o = n0 + 4 * ch;
     if (o >= L.out) return;
     const float4 bv = __ldg(reinterpret_cast<const float4*>(L.bias + o));
     const bool gelu = L.act == CFI_ACT_GELU_ERF;
@@ -117,7 +114,7 @@ __device__ __forceinline__ void sp_reduce(const DevLayer& L, float* __restrict__
 #pragma unroll
         for (int j = 0; j < kRows; ++j) {
             const int b = split * rows_per + rr0 + j * kSpWorkerWarps;
-            if (rr0 + j * kSpWorkerWarps < rows_per && b < BT && b0 + b < batch) {
+            if (rr0 + j * kSpWorkerWarps < rows_per && b < rows && b0 + b < batch) {
                 const uint32_t off = base + (uint32_t)b * 512u + (uint32_t)ch * 16u;
 #pragma unroll
                 for (int p = 0; p < NS; ++p)
@@ -127,7 +124,7 @@ __device__ __forceinline__ void sp_reduce(const DevLayer& L, float* __restrict__
 #pragma unroll
         for (int j = 0; j < kRows; ++j) {
             const int b = split * rows_per + rr0 + j * kSpWorkerWarps;
-            if (rr0 + j * kSpWorkerWarps < rows_per && b < BT && b0 + b < batch) {
+            if (rr0 + j * kSpWorkerWarps < rows_per && b < rows && b0 + b < batch) {
                 float4 a = t[j][0];
 #pragma unroll
                 for (int p = 1; p < NS; ++p) a.x += t[j][p].x, a.y += t[j][p].y, a.z += t[j][p].z, a.w += t[j][p].w;
@@ -151,12 +148,13 @@ __device__ __forceinline__ void sp_reduce(const DevLayer& L, float* __restrict__
 template <int BT>
 __global__ void __launch_bounds__(kSpThreads, 1)
 cfi_dense_split_kernel(DevLayer L, const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x,
-                       float* __restrict__ y, int batch) {
+                       float* __restrict__ y, int batch, int rows) {
     static_assert(BT % 16 == 0 && BT >= 16 && BT <= 128, "batch tile");
     constexpr int kSpStages = sp_stages(BT);
-    constexpr uint32_t kXBytes = sp_x_bytes(BT), kStageBytes = sp_stage_bytes(BT);
-    constexpr uint32_t kABase = kSpTmemCols - 32 * kSpStages;  // accumulators in columns 0 .. 3BT-1, w_lo stages at the top
-    static_assert(3 * BT <= kABase, "tensor memory: accumulators + w_lo stages");
+    constexpr uint32_t kStageBytes = sp_stage_bytes(BT);
+    const uint32_t x_bytes = sp_x_bytes(rows);  // rows <= BT of the tile are in use; x_lo begins behind them
+    constexpr uint32_t kABase = kSpTmemCols - 64 * kSpStages;  // accumulators in columns 0 .. 2 BT - 1, weight stages at the top
+    static_assert(2 * BT <= kABase, "tensor memory: accumulators + weight stages");
     static_assert(kSpStages % kSpTeams == 0 && kSpStages <= 8, "a ring slot belongs to one team; eight barriers of each kind");
     constexpr int kTeam = 32 * kSpTeamWarps;                    // threads that prepare one block
     constexpr int kVec = (BT * (kSpK / 4) + kTeam - 1) / kTeam; // 16-byte pieces of the x box per worker and block
@@ -166,7 +164,7 @@ cfi_dense_split_kernel(DevLayer L, const __grid_constant__ CUtensorMap map_w, co
     const uint32_t ring = base, ctl = base + sp_data_bytes(BT);
     const uint32_t full0 = smem_u32(ctl), ready0 = smem_u32(ctl + 64), empty0 = smem_u32(ctl + 128), accum = smem_u32(ctl + 192);
     volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_at(ctl + 200));
-    const int n0 = blockIdx.x * kSpM, b0 = blockIdx.y * BT;  // first output row and first batch row of the tile
+    const int n0 = blockIdx.x * kSpM, b0 = blockIdx.y * rows;  // first output row and first batch row of the tile
     const int k_blocks = (L.in + kSpK - 1) / kSpK;
     const int split = (int)cluster_rank(), n_split = (int)cluster_size();
     const int kb0 = (int)(((int64_t)k_blocks * split) / n_split);
@@ -187,7 +185,7 @@ cfi_dense_split_kernel(DevLayer L, const __grid_constant__ CUtensorMap map_w, co
         // rest of the set-up and before the wait for the kernel ahead (each stage's barrier already expects the x box
         // as well).
         for (int i = 0; i < n_local && i < kSpStages; ++i) {
-            mbar_expect_tx(full0 + 8 * i, kSpWBytes + kXBytes);
+            mbar_expect_tx(full0 + 8 * i, kSpWBytes + x_bytes);
             tma_load_2d(smem_u32(ring + i * kStageBytes), &map_w, full0 + 8 * i, (kb0 + i) * kSpK, n0);
         }
     }
@@ -219,44 +217,53 @@ cfi_dense_split_kernel(DevLayer L, const __grid_constant__ CUtensorMap map_w, co
             if (i >= kSpStages) {
                 ok = mbar_wait(empty0 + 8 * s, (uint32_t)(i / kSpStages - 1) & 1u, kTcSpinLimit);
                 if (!ok) break;
-                mbar_expect_tx(full0 + 8 * s, kSpWBytes + kXBytes);
+                mbar_expect_tx(full0 + 8 * s, kSpWBytes + x_bytes);
                 tma_load_2d(dst, &map_w, full0 + 8 * s, (kb0 + i) * kSpK, n0);
             }
             tma_load_2d(dst + kSpWBytes, &map_x, full0 + 8 * s, (kb0 + i) * kSpK, b0);
+            // Further on, one CTA of those that read a box asks for it: a trip to DRAM is longer than what the ring holds.
+            const int ahead = i + 2 * kSpStages;
+            if (ahead < n_local) {
+                if (blockIdx.x == 0) tma_prefetch_l2_2d(&map_x, (kb0 + ahead) * kSpK, b0);
+                if (blockIdx.y == 0) tma_prefetch_l2_2d(&map_w, (kb0 + ahead) * kSpK, n0);
+            }
             issued = i + 1;  // (the first ring round has no wait that could fail, so no stage is left with only its weight box)
         }
     } else if (warp == 1 && elect_one()) {
-        // ---------------------------------------------------------------- first MMA issuer: Wd x [x; x_lo], N = 2 BT.
-        // (The two issuers are written out separately: a thread gets a tcgen05 instruction accepted only about every
-        // 150 cycles, and any branch in this loop costs more.  A stage's "ready" barrier completes only after its
-        // "full" barrier has, so one wait covers both.)
-        constexpr uint32_t idesc = sp_instr_desc(2 * BT);
-        for (int i = 0; i < n_local && ok; ++i) {
-            const int s = i % kSpStages;
-            ok = mbar_wait(ready0 + 8 * s, (uint32_t)(i / kSpStages) & 1u, kTcSpinLimit);
-            if (!ok) break;
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t st = smem_u32(ring + s * kStageBytes);
-            const uint64_t dw = umma_desc_k_sw128(st), dx = umma_desc_k_sw128(st + kSpWBytes);
-            umma_tf32_ss(tmem_base, dw, dx, idesc, i != 0 ? 1u : 0u);  // 8 fp32 further along K: 32 bytes of a row
-            umma_tf32_ss(tmem_base, dw + 2u, dx + 2u, idesc, 1u);
-            umma_tf32_ss(tmem_base, dw + 4u, dx + 4u, idesc, 1u);
-            umma_tf32_ss(tmem_base, dw + 6u, dx + 6u, idesc, 1u);
-            umma_commit(empty0 + 8 * s);
-        }
-        umma_commit(accum);  // also after a failed wait: the arrival then tells when the MMAs issued so far are done
-    } else if (warp == 2 && elect_one()) {
-        // ---------------------------------------------------------------- second MMA issuer: w_lo x x, N = BT
-        constexpr uint32_t idesc = sp_instr_desc(BT);
-        const uint32_t acc = tmem_base + (uint32_t)(2 * BT);
+        // ---------------------------------------------------------------- first MMA issuer: w_hi x x into columns 0 .. rows - 1.
+        // A stage's "ready" barrier completes only after its "full" barrier has, so one wait covers both.
+        const uint32_t idesc = sp_instr_desc(rows);
         for (int i = 0; i < n_local && ok; ++i) {
             const int s = i % kSpStages;
             ok = mbar_wait(ready0 + 8 * s, (uint32_t)(i / kSpStages) & 1u, kTcSpinLimit);
             if (!ok) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint64_t dx = umma_desc_k_sw128(smem_u32(ring + s * kStageBytes + kSpWBytes));
-            const uint32_t a_lo = tmem_base + kABase + (uint32_t)(32 * s);  // 8 columns of tensor memory per K step
-            umma_tf32_ts(acc, a_lo, dx, idesc, i != 0 ? 1u : 0u);
+            const uint32_t a_hi = tmem_base + kABase + (uint32_t)(64 * s);  // 8 columns of tensor memory per K step
+            umma_tf32_ts(tmem_base, a_hi, dx, idesc, i != 0 ? 1u : 0u);  // 8 fp32 further along K: 32 bytes of a row
+            umma_tf32_ts(tmem_base, a_hi + 8u, dx + 2u, idesc, 1u);
+            umma_tf32_ts(tmem_base, a_hi + 16u, dx + 4u, idesc, 1u);
+            umma_tf32_ts(tmem_base, a_hi + 24u, dx + 6u, idesc, 1u);
+            umma_commit(empty0 + 8 * s);
+        }
+        umma_commit(accum);  // also after a failed wait: the arrival then tells when the MMAs issued so far are done
+    } else if (warp == 2 && elect_one()) {
+        // ---------------------------------------------------------------- second MMA issuer: w_hi x x_lo + w_lo x x into columns
+        // rows .. 2 rows - 1 (one accumulator, one shape: in order)
+        const uint32_t idesc = sp_instr_desc(rows), acc = tmem_base + (uint32_t)rows;
+        for (int i = 0; i < n_local && ok; ++i) {
+            const int s = i % kSpStages;
+            ok = mbar_wait(ready0 + 8 * s, (uint32_t)(i / kSpStages) & 1u, kTcSpinLimit);
+            if (!ok) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t xs = smem_u32(ring + s * kStageBytes + kSpWBytes);
+            const uint64_t dx = umma_desc_k_sw128(xs), dl = umma_desc_k_sw128(xs + x_bytes);
+            const uint32_t a_hi = tmem_base + kABase + (uint32_t)(64 * s), a_lo = a_hi + 32u;
+            umma_tf32_ts(acc, a_hi, dl, idesc, i != 0 ? 1u : 0u);
+            umma_tf32_ts(acc, a_hi + 8u, dl + 2u, idesc, 1u);
+            umma_tf32_ts(acc, a_hi + 16u, dl + 4u, idesc, 1u);
+            umma_tf32_ts(acc, a_hi + 24u, dl + 6u, idesc, 1u);
+            umma_tf32_ts(acc, a_lo, dx, idesc, 1u);
             umma_tf32_ts(acc, a_lo + 8u, dx + 2u, idesc, 1u);
             umma_tf32_ts(acc, a_lo + 16u, dx + 4u, idesc, 1u);
             umma_tf32_ts(acc, a_lo + 24u, dx + 6u, idesc, 1u);
@@ -282,25 +289,27 @@ cfi_dense_split_kernel(DevLayer L, const __grid_constant__ CUtensorMap map_w, co
 #pragma unroll
             for (int j = 0; j < kVec; ++j) {
                 const uint32_t f = (uint32_t)(wt + j * kTeam) * 16u;
-                if (f < kXBytes) {
+                if (f < x_bytes) {
                     const float4 v = *reinterpret_cast<const float4*>(smem_at(xs + f));
-                    *reinterpret_cast<float4*>(smem_at(xs + kXBytes + f)) = make_float4(tf32_lo(v.x), tf32_lo(v.y), tf32_lo(v.z), tf32_lo(v.w));
+                    *reinterpret_cast<float4*>(smem_at(xs + x_bytes + f)) = make_float4(tf32_lo(v.x), tf32_lo(v.y), tf32_lo(v.z), tf32_lo(v.w));
                 }
             }
-            // w_lo: this thread's half (16 fp32) of output row `row`, un-permuted from the swizzle, into tensor-memory
-            // columns [16 half, 16 half + 16) of the stage.
+            // The weight's two parts: this thread's half (16 fp32) of output row `row`, un-permuted from the swizzle, into
+            // columns 16 half .. 16 half + 15 of the stage's hi and lo columns in tensor memory.
             {
                 const uint32_t row_off = ring + s * kStageBytes + (uint32_t)row * 128u;
-                uint32_t lo[16];
+                uint32_t hi[16], lo[16];
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
                     const float4 w4 = *reinterpret_cast<const float4*>(smem_at(row_off + (uint32_t)(((4 * half + c) ^ (row & 7)) << 4)));
-                    lo[4 * c + 0] = __float_as_uint(tf32_lo(w4.x));
-                    lo[4 * c + 1] = __float_as_uint(tf32_lo(w4.y));
-                    lo[4 * c + 2] = __float_as_uint(tf32_lo(w4.z));
-                    lo[4 * c + 3] = __float_as_uint(tf32_lo(w4.w));
+                    hi[4 * c + 0] = __float_as_uint(w4.x), lo[4 * c + 0] = __float_as_uint(tf32_lo(w4.x));
+                    hi[4 * c + 1] = __float_as_uint(w4.y), lo[4 * c + 1] = __float_as_uint(tf32_lo(w4.y));
+                    hi[4 * c + 2] = __float_as_uint(w4.z), lo[4 * c + 2] = __float_as_uint(tf32_lo(w4.z));
+                    hi[4 * c + 3] = __float_as_uint(w4.w), lo[4 * c + 3] = __float_as_uint(tf32_lo(w4.w));
                 }
-                tmem_st16(tmem_base + ((uint32_t)(32 * q) << 16) + kABase + (uint32_t)(32 * s + 16 * half), lo);
+                const uint32_t a_hi = tmem_base + ((uint32_t)(32 * q) << 16) + kABase + (uint32_t)(64 * s + 16 * half);
+                tmem_st16(a_hi, hi);
+                tmem_st16(a_hi + 32u, lo);
             }
             asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -312,22 +321,22 @@ cfi_dense_split_kernel(DevLayer L, const __grid_constant__ CUtensorMap map_w, co
         if (ok) ok = mbar_wait(accum, 0u, kTcSpinLimit);
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         // The four warps of a lane quarter take the 16-column chunks of the tile in turn.
-        if (ok && 16 * part < BT) {
+        if (ok && 16 * part < rows) {
             const int o = n0 + row;
             auto drain = [&](auto gelu_tag) {
                 constexpr bool kGelu = decltype(gelu_tag)::value;
 #pragma unroll 1
-                for (int c0 = 16 * part; c0 < BT; c0 += 64) {
-                    uint32_t a[3][16];
+                for (int c0 = 16 * part; c0 < rows; c0 += 64) {
+                    uint32_t a[2][16];
                     const uint32_t t = tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)c0;
 #pragma unroll
-                    for (int p = 0; p < 3; ++p) tmem_ld16(t + (uint32_t)(p * BT), a[p]);
+                    for (int p = 0; p < 2; ++p) tmem_ld16(t + (uint32_t)(p * rows), a[p]);
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
                     for (int e = 0; e < 16; ++e) {
                         float sum = 0.0f;
                         if (n_local > 0)  // a CTA without K blocks has issued no MMA: its accumulators hold nothing
-                            sum = (__uint_as_float(a[1][e]) + __uint_as_float(a[2][e])) + __uint_as_float(a[0][e]);
+                            sum = __uint_as_float(a[1][e]) + __uint_as_float(a[0][e]);
                         const int b = c0 + e;
                         if (n_split > 1) {
                             // partial tile [BT][128] fp32: consecutive lanes are consecutive output rows
@@ -349,13 +358,13 @@ cfi_dense_split_kernel(DevLayer L, const __grid_constant__ CUtensorMap map_w, co
         if (warp >= kSpFirstWorker && ok) {
             const int wt = tid - 32 * kSpFirstWorker;
             switch (n_split) {
-                case 2: sp_reduce<BT, 2>(L, y, batch, n0, b0, base, split, wt); break;
-                case 3: sp_reduce<BT, 3>(L, y, batch, n0, b0, base, split, wt); break;
-                case 4: sp_reduce<BT, 4>(L, y, batch, n0, b0, base, split, wt); break;
-                case 5: sp_reduce<BT, 5>(L, y, batch, n0, b0, base, split, wt); break;
-                case 6: sp_reduce<BT, 6>(L, y, batch, n0, b0, base, split, wt); break;
-                case 7: sp_reduce<BT, 7>(L, y, batch, n0, b0, base, split, wt); break;
-                default: sp_reduce<BT, 8>(L, y, batch, n0, b0, base, split, wt); break;
+                case 2: sp_reduce<2>(L, y, batch, n0, b0, rows, base, split, wt); break;
+                case 3: sp_reduce<3>(L, y, batch, n0, b0, rows, base, split, wt); break;
+                case 4: sp_reduce<4>(L, y, batch, n0, b0, rows, base, split, wt); break;
+                case 5: sp_reduce<5>(L, y, batch, n0, b0, rows, base, split, wt); break;
+                case 6: sp_reduce<6>(L, y, batch, n0, b0, rows, base, split, wt); break;
+                case 7: sp_reduce<7>(L, y, batch, n0, b0, rows, base, split, wt); break;
+                default: sp_reduce<8>(L, y, batch, n0, b0, rows, base, split, wt); break;
             }
         }
         cluster_sync_all_relaxed();  // no CTA leaves while another may still read its tile

@@ -928,8 +928,11 @@ constexpr int kMaxSplit = kMaxClusterSplit;
 // wave pays it again), the cluster reduction when K is split, and the launch itself.  The dense weight pieces
 // (4 bytes per dense entry) have to come from HBM at least once per call.
 constexpr double kSplitLaunch = 0.7e-6, kSplitWave = 4.2e-6, kSplitHbmBytesPerSecond = 5.5e12;
-double split_seconds_per_block(int bt) { return bt >= 128 ? 0.51e-6 : bt >= 96 ? 0.40e-6 : 0.31e-6; }  // the issue of 4 + 4 MMAs and a commit
-double split_seconds_reduce(int bt) { return 0.5e-6 + 0.95e-6 * bt / 128.0; }
+double split_seconds_per_block(int rows) {  // by 16 rows of the batch tile
+    constexpr double us[] = {0.22, 0.23, 0.25, 0.26, 0.33, 0.38, 0.43, 0.46};
+    return us[rows / kSpRowStep - 1] * 1e-6;
+}
+double split_seconds_reduce(int rows) { return 0.5e-6 + 0.95e-6 * rows / 128.0; }
 int split_bt_index(int bt) {
     for (int i = 0; i < kSpNumTiles; ++i)
         if (kSpTiles[i] == bt) return i;
@@ -981,7 +984,8 @@ int split_resident_clusters(const cfi_layer* l, int bt, int split) {
 }
 
 struct SplitShape {
-    int bt;          // batch rows per tile: one of kSpTiles (the MMA's N is twice that)
+    int bt;          // batch rows per tile: one of kSpTiles
+    int rows;        // of which each tile uses so many
     int split;       // CTAs per output tile (cluster size along z): 1 .. 8
     double seconds;  // modelled time of the launch
     bool ok;
@@ -993,10 +997,11 @@ struct SplitShape {
 SplitShape split_shape(const cfi_layer* l, int batch, int force_bt = 0, int force_split = 0) {
     const int k_blocks = (l->d.in + kSpK - 1) / kSpK, tiles_m = (l->d.out + kSpM - 1) / kSpM;
     const double t_hbm = 4.0 * l->out_pad * (double)l->d.in / kSplitHbmBytesPerSecond;
-    SplitShape best{128, 1, 0.0, false};
-    for (int bt : kSpTiles) {
-        if (force_bt && bt != force_bt) continue;
-        const int64_t tiles_b = (batch + bt - 1) / bt;
+    SplitShape best{128, 128, 1, 0.0, false};
+    for (int rows = kSpRowStep; rows <= 128; rows += kSpRowStep) {
+        if (force_bt && rows != force_bt) continue;
+        const int bt = *std::lower_bound(std::begin(kSpTiles), std::end(kSpTiles), rows);
+        const int64_t tiles_b = (batch + rows - 1) / rows;
         if (tiles_b > 65535) continue;
         const int64_t tiles = tiles_m * tiles_b;
         for (int split = 1; split <= kMaxSplit; ++split) {
@@ -1004,22 +1009,22 @@ SplitShape split_shape(const cfi_layer* l, int batch, int force_bt = 0, int forc
             const int64_t resident = split_resident_clusters(l, bt, split);
             if (resident == 0) continue;
             const int64_t waves = (tiles + resident - 1) / resident;
-            const double main = (double)waves * ((k_blocks + split - 1) / split) * split_seconds_per_block(bt);
-            const double t = std::max(main, t_hbm) + (double)waves * (kSplitWave + (split > 1 ? split_seconds_reduce(bt) : 0.0)) + kSplitLaunch;
-            if (!best.ok || t < best.seconds) best = SplitShape{bt, split, t, true};
+            const double main = (double)waves * ((k_blocks + split - 1) / split) * split_seconds_per_block(rows);
+            const double t = std::max(main, t_hbm) + (double)waves * (kSplitWave + (split > 1 ? split_seconds_reduce(rows) : 0.0)) + kSplitLaunch;
+            if (!best.ok || t < best.seconds) best = SplitShape{bt, rows, split, t, true};
         }
     }
     return best;
 }
 
 template <int BT>
-cfi_status_t launch_dense_split_bt(const cfi_layer* l, int split, const void* x, void* y, int batch, cudaStream_t st) {
-    const int grid_x = (l->d.out + kSpM - 1) / kSpM, grid_y = (batch + BT - 1) / BT;
-    CUtensorMap map_x;  // x in boxes of BT rows x 32 columns
-    if (!encode_map(&map_x, x, (uint64_t)batch, (uint64_t)l->d.in, 4, BT)) return CFI_ERR_SHAPE;
+cfi_status_t launch_dense_split_bt(const cfi_layer* l, const SplitShape& sh, const void* x, void* y, int batch, cudaStream_t st) {
+    const int grid_x = (l->d.out + kSpM - 1) / kSpM, grid_y = (batch + sh.rows - 1) / sh.rows, split = sh.split;
+    CUtensorMap map_x;  // x in boxes of the tile's rows x 32 columns
+    if (!encode_map(&map_x, x, (uint64_t)batch, (uint64_t)l->d.in, 4, sh.rows)) return CFI_ERR_SHAPE;
     if (cfi_status_t e = set_smem<cfi_dense_split_kernel<BT>>(sp_smem_bytes(BT), l->device)) return e;
     return launch_pdl_cluster(cfi_dense_split_kernel<BT>, dim3(grid_x, grid_y, split), kSpThreads, sp_smem_bytes(BT), split, st, l->d,
-                              l->map_w, map_x, static_cast<float*>(y), batch);
+                              l->map_w, map_x, static_cast<float*>(y), batch, sh.rows);
 }
 
 cfi_status_t launch_dense_split(const cfi_layer* l, const void* x, void* y, int batch, cudaStream_t st, int force_bt = 0,
@@ -1029,12 +1034,12 @@ cfi_status_t launch_dense_split(const cfi_layer* l, const void* x, void* y, int 
     const SplitShape sh = split_shape(l, batch, force_bt, force_split);
     if (!sh.ok) return CFI_ERR_SHAPE;
     switch (sh.bt) {
-        case 16: return launch_dense_split_bt<16>(l, sh.split, x, y, batch, st);
-        case 32: return launch_dense_split_bt<32>(l, sh.split, x, y, batch, st);
-        case 48: return launch_dense_split_bt<48>(l, sh.split, x, y, batch, st);
-        case 64: return launch_dense_split_bt<64>(l, sh.split, x, y, batch, st);
-        case 96: return launch_dense_split_bt<96>(l, sh.split, x, y, batch, st);
-        default: return launch_dense_split_bt<128>(l, sh.split, x, y, batch, st);
+        case 16: return launch_dense_split_bt<16>(l, sh, x, y, batch, st);
+        case 32: return launch_dense_split_bt<32>(l, sh, x, y, batch, st);
+        case 48: return launch_dense_split_bt<48>(l, sh, x, y, batch, st);
+        case 64: return launch_dense_split_bt<64>(l, sh, x, y, batch, st);
+        case 96: return launch_dense_split_bt<96>(l, sh, x, y, batch, st);
+        default: return launch_dense_split_bt<128>(l, sh, x, y, batch, st);
     }
 }
 

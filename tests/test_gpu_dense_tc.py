@@ -55,6 +55,23 @@ def test_dense_split_tf32_every_launch_shape(tile, cluster):
         assert np.array_equal(y, y2)                      # fixed order of additions: the same bits every time
 
 
+@pytest.mark.parametrize("in_f,out_f,k,nabl,B,act", [(512, 384, 51, 9, 797, "none"), (512, 384, 51, 9, 1185, "gelu"),
+                                                      (512, 384, 51, 0, 1641, "none"), (1000, 72, 100, 5, 1677, "gelu"),
+                                                      (1000, 72, 100, 5, 2277, "none"), (520, 640, 52, 30, 2063, "gelu")])
+def test_dense_split_tf32_tiles_used_in_part(in_f, out_f, k, nabl, B, act):
+    """Batches for which the library takes 80 of a tile's 96 rows or 112 of 128, with and without a K split, ragged at every edge."""
+    from paper_2305_02299_b200 import binding as cfi
+    L = inputs.make_layer(in_f, out_f, k, n_ablated=nabl, seed=in_f + B)
+    x = inputs.make_x(B, in_f, seed=B)
+    y_ref, S = oracle_layer(L, x, "f32", act)
+    dl = device_layer(L, "f32", act)
+    assert cfi.cfi_dense_tile_shape(dl, B)[0] in (96, 128)
+    y = run_device(dl, x, "f32", "dense_tc")
+    assert cfi.cfi_device_status(dl) == 0
+    dl.close()
+    assert scaled_error(y, y_ref, S) <= TOL["f32"]
+
+
 @pytest.mark.parametrize("tile,cluster", [(16, 4), (48, 4), (64, 8), (96, 2), (128, 2), (32, 1)])
 def test_dense_split_tf32_chain_of_launches(tile, cluster):
     """Back-to-back launches (a CUDA graph of 48 calls over 6 rotating layers; each launch lets its successor start
