@@ -64,6 +64,7 @@ constexpr int kSpRowStep = 16;
 // The depth is a multiple of the number of worker teams, so that a ring slot always belongs to the same team: a team
 // that met only every other phase of a slot's barrier could not tell a phase from the one two before it by parity.
 __host__ __device__ constexpr int sp_stages(int bt) { return bt >= 96 ? 4 : 6; }
+constexpr int kSpLeft = 1 << 30;     // more than any number of K blocks (2^26 at most), with room to add to
 constexpr int kMaxClusterSplit = 8;  // largest portable thread-block cluster
 constexpr uint32_t kSpWBytes = kSpM * kSpK * 4;  // one weight box: 16 KB
 constexpr uint32_t kSpTmemCols = 512;            // 2 BT accumulator columns ... one stage of 2 x 32 weight columns per ring slot at the top
@@ -165,7 +166,7 @@ cfi_dense_split_kernel(DevLayer L, const __grid_constant__ CUtensorMap map_w, co
     const uint32_t ring = base, ctl = base + sp_data_bytes(BT);
     const uint32_t full0 = smem_u32(ctl), ready0 = smem_u32(ctl + 64), empty0 = smem_u32(ctl + 128), accum = smem_u32(ctl + 192);
     volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_at(ctl + 200));
-    volatile int* progress = reinterpret_cast<volatile int*>(smem_at(ctl + 204));  // blocks the TMA lane has come to; INT_MAX: it has left
+    volatile int* progress = reinterpret_cast<volatile int*>(smem_at(ctl + 204));  // blocks the TMA lane has come to; kSpLeft: it has left
     const int n0 = blockIdx.x * kSpM, b0 = blockIdx.y * rows;  // first output row and first batch row of the tile
     const int k_blocks = (L.in + kSpK - 1) / kSpK;
     const int split = (int)cluster_rank(), n_split = (int)cluster_size();
@@ -220,7 +221,7 @@ cfi_dense_split_kernel(DevLayer L, const __grid_constant__ CUtensorMap map_w, co
             *progress = i + 1;
             issued = i + 1;  // (the first ring round has no wait that could fail, so no stage is left with only its weight box)
         }
-        *progress = 0x7fffffff;
+        *progress = kSpLeft;
     } else if (warp == 3 && lane == 0) {
         // ---------------------------------------------------------------- L2 prefetch, by one CTA of those that read a box.
         // x may belong to the kernel ahead and must not be read before that kernel is done; asking for its boxes to be
@@ -231,7 +232,7 @@ cfi_dense_split_kernel(DevLayer L, const __grid_constant__ CUtensorMap map_w, co
         const bool ask_x = blockIdx.x == 0, ask_w = blockIdx.y == 0;
         for (int i = 0, polls = 0; i < n_local && (ask_x || ask_w); ++i) {
             while (*progress + 2 * kSpStages <= i && polls < (int)kTcSpinLimit) ++polls, __nanosleep(100);
-            if (*progress == 0x7fffffff || polls >= (int)kTcSpinLimit) break;
+            if (*progress == kSpLeft || polls >= (int)kTcSpinLimit) break;
             if (ask_x) tma_prefetch_l2_2d(&map_x, (kb0 + i) * kSpK, b0);
             if (ask_w && i >= kSpStages) tma_prefetch_l2_2d(&map_w, (kb0 + i) * kSpK, n0);
         }

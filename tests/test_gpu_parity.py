@@ -38,6 +38,16 @@ def test_odd_shapes(in_f, out_f, k, dtype):
         check_layer(L, inputs.make_x(B, in_f, seed=3), dtype, variants=ALL)
 
 
+@pytest.mark.parametrize("in_f,out_f,k", [(8, 40, 3), (2918, 64, 280), (3333, 24, 2000), (4096, 40, 3000), (4100, 33, 1)])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_small_batch_rows_of_x(in_f, out_f, k, dtype):
+    """The small-batch kernel's copies of x (rows of whole 16-byte pieces, of 4-byte words, of odd bf16 length), its batch tiles
+    of 1, 2, 4 and 8 full and in part, and rows longer than what a group of lanes has in flight."""
+    L = inputs.make_layer(in_f, out_f, k, n_ablated=out_f // 9, seed=in_f)
+    for B in (1, 2, 3, 4, 5, 8, 11):
+        check_layer(L, inputs.make_x(B, in_f, seed=B), dtype, variants=("splitk",))
+
+
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("act", ["none", "gelu"])
 def test_gelu_and_ablated_rows(dtype, act):
