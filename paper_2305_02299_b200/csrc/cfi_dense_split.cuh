@@ -22,7 +22,7 @@
 //
 // The layer keeps one dense fp32 copy of its weight, Wd[out_pad][in] (zero rows for ablated and padding rows).  A tile
 // is 128 output rows (M) x BT batch rows (N side), so a small batch costs a narrow MMA and not a mostly empty 128-row
-// tile.  Per 32-column block of K, in a ring of four or six stages [Wd box | x box | x_lo]:
+// tile.  Per 32-column block of K, in a ring of four to eight stages [Wd box | x box | x_lo]:
 //   warp 0, one lane    TMA: the 128 x 32 box of Wd and the BT x 32 box of x (fp32, 128-byte swizzle).  The weight
 //                       boxes of the first ring round are requested before the wait for the kernel ahead;
 //   warps 4..19         two teams of eight worker warps; team t prepares the blocks i = t (mod 2).  x_lo: the x box is
@@ -55,7 +55,7 @@ constexpr int kSpM = 128, kSpK = 32;
 constexpr int kSpTeamWarps = 8, kSpTeams = 2, kSpWorkerWarps = kSpTeams * kSpTeamWarps, kSpFirstWorker = 4;
 constexpr int kSpThreads = 32 * (kSpFirstWorker + kSpWorkerWarps);
 // Batch tiles of the kernel (the MMA's N is BT, a multiple of 16) and the ring depth each one affords in shared memory
-// (16 KB + 256 BT bytes per stage) and tensor memory (2 BT accumulator columns + 64 per stage).
+// (16 KB + 256 BT bytes per stage).  Tensor memory: 2 BT accumulator columns + 64 per weight stage.
 constexpr int kSpTiles[] = {16, 32, 48, 64, 96, 128};
 constexpr int kSpNumTiles = sizeof(kSpTiles) / sizeof(kSpTiles[0]);
 // A launch may use fewer rows of its tiles, in steps of 16 (the MMA's N): 80 of 96, or 112 of 128, where that fills the SMs
@@ -63,7 +63,10 @@ constexpr int kSpNumTiles = sizeof(kSpTiles) / sizeof(kSpTiles[0]);
 constexpr int kSpRowStep = 16;
 // The depth is a multiple of the number of worker teams, so that a ring slot always belongs to the same team: a team
 // that met only every other phase of a slot's barrier could not tell a phase from the one two before it by parity.
-__host__ __device__ constexpr int sp_stages(int bt) { return bt >= 96 ? 4 : 6; }
+__host__ __device__ constexpr int sp_stages(int bt) { return bt >= 96 ? 4 : bt >= 48 ? 6 : 8; }
+// Weight stages in tensor memory: fewer than the ring has where the tile is narrow and the call a stream of weight boxes, for
+// which the ring is as deep as it gets (cold 4096 x 4096 at batch 16: 15.8 us with six slots, 15.25 with eight).
+__host__ __device__ constexpr int sp_weight_stages(int bt) { return bt >= 96 ? 4 : 6; }
 constexpr int kSpLeft = 1 << 30;     // more than any number of K blocks (2^26 at most), with room to add to
 constexpr int kMaxClusterSplit = 8;  // largest portable thread-block cluster
 constexpr uint32_t kSpWBytes = kSpM * kSpK * 4;  // one weight box: 16 KB
@@ -152,12 +155,12 @@ __global__ void __launch_bounds__(kSpThreads, 1)
 cfi_dense_split_kernel(DevLayer L, const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x,
                        float* __restrict__ y, int batch, int rows) {
     static_assert(BT % 16 == 0 && BT >= 16 && BT <= 128, "batch tile");
-    constexpr int kSpStages = sp_stages(BT);
+    constexpr int kSpStages = sp_stages(BT), kWStages = sp_weight_stages(BT);
     constexpr uint32_t kStageBytes = sp_stage_bytes(BT);
     const uint32_t x_bytes = sp_x_bytes(rows);  // rows <= BT of the tile are in use; x_lo begins behind them
-    constexpr uint32_t kABase = kSpTmemCols - 64 * kSpStages;  // accumulators in columns 0 .. 2 BT - 1, weight stages at the top
+    constexpr uint32_t kABase = kSpTmemCols - 64 * kWStages;  // accumulators in columns 0 .. 2 BT - 1, weight stages at the top
     static_assert(2 * BT <= kABase, "tensor memory: accumulators + weight stages");
-    static_assert(kSpStages % kSpTeams == 0 && kSpStages <= 8, "a ring slot belongs to one team; eight barriers of each kind");
+    static_assert(kSpStages % kSpTeams == 0 && kWStages % kSpTeams == 0 && kWStages <= kSpStages && kSpStages <= 8, "a ring slot belongs to one team; eight barriers of each kind");
     constexpr int kTeam = 32 * kSpTeamWarps;                    // threads that prepare one block
     constexpr int kVec = (BT * (kSpK / 4) + kTeam - 1) / kTeam; // 16-byte pieces of the x box per worker and block
     pdl_launch_dependents();
@@ -246,7 +249,7 @@ cfi_dense_split_kernel(DevLayer L, const __grid_constant__ CUtensorMap map_w, co
             if (!ok) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint64_t dx = umma_desc_k_sw128(smem_u32(ring + s * kStageBytes + kSpWBytes));
-            const uint32_t a_hi = tmem_base + kABase + (uint32_t)(64 * s);  // 8 columns of tensor memory per K step
+            const uint32_t a_hi = tmem_base + kABase + (uint32_t)(64 * (i % kWStages));  // 8 columns of tensor memory per K step
             umma_tf32_ts(tmem_base, a_hi, dx, idesc, i != 0 ? 1u : 0u);  // 8 fp32 further along K: 32 bytes of a row
             umma_tf32_ts(tmem_base, a_hi + 8u, dx + 2u, idesc, 1u);
             umma_tf32_ts(tmem_base, a_hi + 16u, dx + 4u, idesc, 1u);
@@ -265,7 +268,7 @@ cfi_dense_split_kernel(DevLayer L, const __grid_constant__ CUtensorMap map_w, co
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint32_t xs = smem_u32(ring + s * kStageBytes + kSpWBytes);
             const uint64_t dx = umma_desc_k_sw128(xs), dl = umma_desc_k_sw128(xs + x_bytes);
-            const uint32_t a_hi = tmem_base + kABase + (uint32_t)(64 * s), a_lo = a_hi + 32u;
+            const uint32_t a_hi = tmem_base + kABase + (uint32_t)(64 * (i % kWStages)), a_lo = a_hi + 32u;
             umma_tf32_ts(acc, a_hi, dl, idesc, i != 0 ? 1u : 0u);
             umma_tf32_ts(acc, a_hi + 8u, dl + 2u, idesc, 1u);
             umma_tf32_ts(acc, a_hi + 16u, dl + 4u, idesc, 1u);
@@ -303,6 +306,12 @@ cfi_dense_split_kernel(DevLayer L, const __grid_constant__ CUtensorMap map_w, co
             }
             // The weight's two parts: this thread's half (16 fp32) of output row `row`, un-permuted from the swizzle, into
             // columns 16 half .. 16 half + 15 of the stage's hi and lo columns in tensor memory.
+            if (kWStages < kSpStages && i >= kWStages) {  // the MMAs that read the stage's columns last are done
+                const int b = i - kWStages;
+                ok = mbar_wait(empty0 + 8 * (b % kSpStages), (uint32_t)(b / kSpStages) & 1u, kTcSpinLimit);
+                if (!ok) break;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            }
             {
                 const uint32_t row_off = ring + s * kStageBytes + (uint32_t)row * 128u;
                 uint32_t hi[16], lo[16];
@@ -314,7 +323,7 @@ cfi_dense_split_kernel(DevLayer L, const __grid_constant__ CUtensorMap map_w, co
                     hi[4 * c + 2] = __float_as_uint(w4.z), lo[4 * c + 2] = __float_as_uint(tf32_lo(w4.z));
                     hi[4 * c + 3] = __float_as_uint(w4.w), lo[4 * c + 3] = __float_as_uint(tf32_lo(w4.w));
                 }
-                const uint32_t a_hi = tmem_base + ((uint32_t)(32 * q) << 16) + kABase + (uint32_t)(64 * s + 16 * half);
+                const uint32_t a_hi = tmem_base + ((uint32_t)(32 * q) << 16) + kABase + (uint32_t)(64 * (i % kWStages) + 16 * half);
                 tmem_st16(a_hi, hi);
                 tmem_st16(a_hi + 32u, lo);
             }
