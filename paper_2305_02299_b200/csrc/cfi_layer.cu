@@ -684,7 +684,7 @@ SplitkShape splitk_shape(const cfi_layer* l, int batch) {
     // also limits how many CTAs fit an SM; the grid is sized to one wave of what fits (at most eight CTAs per
     // SM), with several rows per group when needed (rows of a group run one after the other).
     s.smem = smem_of(s.bt);
-    s.grid_y = (batch + s.bt - 1) / s.bt;
+    s.grid_y = std::max(1, (batch + s.bt - 1) / s.bt);  // (a layer without outputs and a batch of none have a shape too: it is asked for, not launched)
     const int fit = (int)std::max<size_t>(1, std::min<size_t>(8, ((size_t)227 * 1024) / (s.smem + 1024)));
     const int64_t lanes = (int64_t)l->d.out * s.g;
     if (splitk_by_rows(l, s.bt)) {
@@ -693,7 +693,7 @@ SplitkShape splitk_shape(const cfi_layer* l, int batch) {
         const int64_t lanes_per_sm = (lanes * s.grid_y + l->sm_count - 1) / l->sm_count;
         const int per_sm = (int)std::max<int64_t>(1, std::min<int64_t>({fit, 4, (lanes_per_sm + 511) / 512}));
         const int slots = std::max(1, l->sm_count * per_sm / s.grid_y);
-        const int rows = (l->d.out + slots - 1) / slots, at_once = 512 / s.g, warp_rows = 32 / s.g;
+        const int rows = std::max(1, (l->d.out + slots - 1) / slots), at_once = 512 / s.g, warp_rows = 32 / s.g;
         s.rows_per_group = (rows + at_once - 1) / at_once;
         int groups = (rows + s.rows_per_group - 1) / s.rows_per_group;
         groups = std::max((groups + warp_rows - 1) / warp_rows * warp_rows, 128 / s.g);

@@ -103,6 +103,25 @@ def test_batch_zero_launches_nothing():
 
 
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("layouts", [1, 3, 7])
+def test_layer_without_outputs(dtype, layouts):
+    """The compact form of a layer whose neurons are all ablated: it can be asked for its kernel and run, at no work at all."""
+    import torch
+    from paper_2305_02299_b200 import binding as cfi
+    empty = cfi.cfi_create(np.zeros((0, 0), np.float32), np.zeros((0, 0), np.int32), np.zeros((0,), np.int32), None, 24, 0, dtype=dtype, layouts=layouts)
+    L = inputs.make_layer(24, 8, 3, seed=0)
+    full = cfi.cfi_create(*cfi.cfi_pack(L.w_dense, L.mask), None, 24, 8, dtype=dtype, layouts=layouts)
+    for B in (0, 1, 2, 16, 32, 300):
+        assert cfi.cfi_choose_variant(empty, B) in (1, 2, 3, 4, 5)
+        assert cfi.cfi_choose_variant(full, B) in (1, 2, 3, 4, 5)
+        x = torch.zeros((B, 24), device="cuda", dtype=torch_dtype(dtype))
+        cfi.cfi_forward(empty, x, torch.empty((16,), device="cuda", dtype=torch_dtype(dtype)), B)
+    assert cfi.cfi_device_status(empty) == 0
+    empty.close()
+    full.close()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("B", [1, 6, 40, 130])
 def test_exact_integer_arithmetic_is_bit_exact(dtype, B):
     """Small-integer weights and inputs: every partial sum is exact in fp32 (and every output fits bf16
