@@ -191,9 +191,10 @@ cfi_status_t cfi_pack_device(const float* w_dense, const uint8_t* mask, int32_t 
 
 /*
  * cfi_pack_device_fill — the arrays of a layer whose size query (cfi_pack_device with NULL arrays) has just been made with
- * the same mask and workspace, both untouched since: the rows are not counted again.  k and n_active are what the query
- * returned, both at least 1; where the workspace holds other counts nothing is written.  Waits for `stream`.  Errors as
- * cfi_pack_device.
+ * the same mask and workspace, both untouched since: the rows are not ranked again.  k and n_active are what the query
+ * returned, both at least 1.  Where the workspace holds other counts nothing is written and the call returns CFI_ERR_SHAPE;
+ * where a row of the mask keeps another number of weights than at the query, CFI_ERR_NOT_CONSTANT_FAN_IN, and the arrays
+ * (written nowhere beyond their ends) are of no use until the next query.  Waits for `stream`.  Other errors as cfi_pack_device.
  */
 cfi_status_t cfi_pack_device_fill(const float* w_dense, const uint8_t* mask, int32_t out_features, int32_t in_features,
                                   void* workspace, size_t workspace_bytes, int32_t k, int32_t n_active, float* values,

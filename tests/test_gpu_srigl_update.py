@@ -216,7 +216,7 @@ def test_pack_device_errors_and_empty():
 
 
 def test_pack_device_fill_writes_only_what_was_counted():
-    """The filling step takes the counts of the size query; with other counts it writes nothing."""
+    """The filling step takes the counts of the size query; with other counts it writes nothing and says so."""
     import ctypes
     import torch
     from paper_2305_02299_b200 import binding as cfi
@@ -233,13 +233,44 @@ def test_pack_device_fill_writes_only_what_was_counted():
     ix, rows = torch.full((out_f, in_f), -1, dtype=torch.int32, device="cuda"), torch.full((out_f,), -1, dtype=torch.int32, device="cuda")
     arrays = (v.data_ptr(), ix.data_ptr(), rows.data_ptr(), None)
     for wrong in ((k - 1, out_f - 3), (k, out_f - 4), (k + 1, out_f - 3)):
-        assert cfi._lib.cfi_pack_device_fill(*head, *wrong, *arrays) == 0
+        assert cfi._lib.cfi_pack_device_fill(*head, *wrong, *arrays) == 2
         assert bool((v == -1).all()) and bool((ix == -1).all()) and bool((rows == -1).all())
     assert cfi._lib.cfi_pack_device_fill(*head, k, out_f - 3, *arrays) == 0
     hv, hix, hrows = cfi.cfi_pack(L.w_dense, L.mask)
     n = hv.size
     assert np.array_equal(v.flatten()[:n].cpu().numpy(), hv.ravel()) and np.array_equal(ix.flatten()[:n].cpu().numpy(), hix.ravel())
     assert np.array_equal(rows[:out_f - 3].cpu().numpy(), hrows) and bool((v.flatten()[n:] == -1).all())
+
+
+@pytest.mark.parametrize("in_f", [96, 99])
+@pytest.mark.parametrize("change", ["fewer", "more", "moved", "empty_row"])
+def test_pack_device_fill_reports_a_mask_that_changed_since_the_query(in_f, change):
+    """A mask that another stream changes between the two steps: never a success with arrays that were not filled."""
+    import ctypes
+    import torch
+    from paper_2305_02299_b200 import binding as cfi
+    out_f, k = 40, 7
+    L = inputs.make_layer(in_f, out_f, k, n_ablated=3, seed=6)
+    w, m = torch.from_numpy(L.w_dense).cuda(), torch.from_numpy(L.mask).cuda()
+    ws = torch.empty(8 * out_f + 512, dtype=torch.uint8, device="cuda")
+    base = (ws.data_ptr() + 255) & ~255
+    kk, na = ctypes.c_int32(0), ctypes.c_int32(0)
+    head = (w.data_ptr(), m.data_ptr(), out_f, in_f, base, 8 * out_f + 256)
+    query = lambda: cfi._lib.cfi_pack_device(*head, ctypes.byref(kk), ctypes.byref(na), None, None, None, None)
+    assert query() == 0 and (kk.value, na.value) == (k, out_f - 3)
+    counts = m.sum(1)
+    row, other, empty = (int(counts.nonzero()[0]), int(counts.nonzero()[1]), int((counts == 0).nonzero()[0]))
+    if change != "more":
+        m[row, m[row].nonzero()[0]] = 0
+    if change != "fewer":
+        to = {"more": row, "moved": other, "empty_row": empty}[change]
+        m[to, (m[to] == 0).nonzero()[-1]] = 1
+    guard = 64
+    v = torch.full(((out_f - 3) * k + guard,), -1.0, device="cuda")
+    ix, rows = torch.full(v.shape, -1, dtype=torch.int32, device="cuda"), torch.full((out_f - 3 + guard,), -1, dtype=torch.int32, device="cuda")
+    assert cfi._lib.cfi_pack_device_fill(*head, k, out_f - 3, v.data_ptr(), ix.data_ptr(), rows.data_ptr(), None) == 3
+    assert bool((v[-guard:] == -1).all()) and bool((ix[-guard:] == -1).all()) and bool((rows[-guard:] == -1).all())
+    assert query() == 3                                           # as the rows are counted anew
 
 
 @pytest.mark.parametrize("in_f", [132, 768, 1030, 4096])
