@@ -201,6 +201,19 @@ def test_pack_device_equals_host_pack(out_f, in_f, k, n_abl):
     assert np.array_equal(vh, vo) and np.array_equal(ih, io) and np.array_equal(rh, ro)
 
 
+@pytest.mark.parametrize("in_f", [1, 31, 511, 512, 513, 1025, 9001])
+def test_pack_device_rows_without_wide_loads(in_f):
+    """Rows whose mask cannot be read 16 bytes at a time (odd lengths; 512 from an odd address): around the 512 columns of a step."""
+    import torch
+    from paper_2305_02299_b200 import binding as cfi
+    w, m, _ = _layer(9, in_f, max(1, in_f // 5), 1, seed=in_f)
+    m_d = torch.empty(m.size + 1, dtype=torch.uint8, device="cuda")[1:].view(m.shape)
+    m_d.copy_(torch.from_numpy(m))
+    v, ix, rows = cfi.cfi_pack_device(torch.from_numpy(w).cuda(), m_d)
+    vh, ih, rh = cfi.cfi_pack(w, m)
+    assert np.array_equal(v.cpu().numpy(), vh) and np.array_equal(ix.cpu().numpy(), ih) and np.array_equal(rows.cpu().numpy(), rh)
+
+
 def test_pack_device_errors_and_empty():
     import torch
     from paper_2305_02299_b200 import binding as cfi
