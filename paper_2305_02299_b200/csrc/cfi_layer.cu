@@ -669,13 +669,20 @@ int splitk_lanes_per_row(int nvec, int units) {
 // fp32 at batch 1 stages x with plain 16-byte loads (cfi_splitk_kernel), everything else row by row (cfi_splitk_rows_kernel).
 bool splitk_by_rows(const cfi_layer* l, int bt) { return l->dtype == CFI_BF16 || bt > 1; }
 
+// Rows of x per tile.  A narrow tile takes fewer lanes a row (splitk_rows_units), leaves more CTAs to a small layer and has
+// less to stage before its first product, a wide one reads the weights (from L2, after the first tile) less often.  Measured
+// over 17 widths, 80 .. 99 % sparsity, fp32 and bf16, against the fastest of tiles of 2, 4 and 8, geometric mean: batch 3 and 4
+// 1.01 .. 1.02 with tiles of 2, 1.2 with one of 4; batch 5 .. 64 1.01 .. 1.04 with 4, 1.25 .. 1.12 with 8; batch 96 and 128
+// 1.04 .. 1.06 and 1.09; batch 197 and 256 1.12 .. 1.17 with 4, 1.06 .. 1.08 with 8.
+int splitk_batch_tile(int batch) { return batch > 128 ? 8 : batch >= 5 ? 4 : batch >= 2 ? 2 : 1; }
+
 SplitkShape splitk_shape(const cfi_layer* l, int batch) {
     SplitkShape s{};
     const int es = l->dtype == CFI_BF16 ? 2 : 4;
     auto smem_of = [&](int bt) {
         return splitk_by_rows(l, bt) ? (size_t)splitk_rows_pitch(l->d.in, es) * bt * es : (size_t)(l->d.in + 1) * bt * 4;
     };
-    s.bt = batch >= 5 ? 8 : batch >= 3 ? 4 : batch == 2 ? 2 : 1;
+    s.bt = splitk_batch_tile(batch);
     while (s.bt > 1 && smem_of(s.bt) > (size_t)l->smem_optin) s.bt >>= 1;
     const int nvec = l->d.kp / vec_of(l->dtype, l->d.idx16 != 0);
     s.g = splitk_lanes_per_row(nvec, splitk_by_rows(l, s.bt) ? splitk_rows_units(l->dtype == CFI_F32, l->d.idx16 != 0, s.bt)
@@ -689,9 +696,11 @@ SplitkShape splitk_shape(const cfi_layer* l, int batch) {
     const int64_t lanes = (int64_t)l->d.out * s.g;
     if (splitk_by_rows(l, s.bt)) {
         // As few CTAs per SM as give every lane a row (at most 512 lanes each, what fits beside the staged x), the rows
-        // spread evenly over them: 5.2 rows of 768 on each of 148 SMs rather than 16 rows on 48.
+        // spread evenly over them: 5.2 rows of 768 on each of 148 SMs rather than 16 rows on 48.  No more than the registers
+        // let an SM hold (two of 64 a thread; tiles of 1 and 2 rows take up to 82): a CTA that has to wait for another to end
+        // stages x all over (768 -> 3072 at batch 16: 7.5 us with three, 4.5 with two).
         const int64_t lanes_per_sm = (lanes * s.grid_y + l->sm_count - 1) / l->sm_count;
-        const int per_sm = (int)std::max<int64_t>(1, std::min<int64_t>({fit, 4, (lanes_per_sm + 511) / 512}));
+        const int per_sm = (int)std::max<int64_t>(1, std::min<int64_t>({fit, s.bt >= 4 ? 2 : 1, (lanes_per_sm + 511) / 512}));
         const int slots = std::max(1, l->sm_count * per_sm / s.grid_y);
         const int rows = std::max(1, (l->d.out + slots - 1) / slots), at_once = 512 / s.g, warp_rows = 32 / s.g;
         s.rows_per_group = (rows + at_once - 1) / at_once;

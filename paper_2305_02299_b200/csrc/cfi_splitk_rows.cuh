@@ -31,7 +31,7 @@ __host__ __device__ constexpr int splitk_rows_units(bool fp32_values, bool idx16
 }
 
 template <typename VT, bool I16, int BT, int G>
-__global__ void __launch_bounds__(512) cfi_splitk_rows_kernel(DevLayer L, const VT* __restrict__ x, VT* __restrict__ y, int batch, int rows_per_group) {
+__global__ void __launch_bounds__(512, BT >= 4 ? 2 : 1) cfi_splitk_rows_kernel(DevLayer L, const VT* __restrict__ x, VT* __restrict__ y, int batch, int rows_per_group) {
     using CK = Chunk<VT, I16>;
     constexpr uint32_t kIdxBytes = I16 ? 2 : 4;
     constexpr int U = splitk_rows_units(sizeof(VT) == 4, I16, BT);
