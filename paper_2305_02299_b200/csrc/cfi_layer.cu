@@ -1259,47 +1259,57 @@ int fallback_variant(const cfi_layer* l, int batch) {
     return CFI_VARIANT_SIMPLE;
 }
 
-// Time model of the slab kernel (measured, fp32): a fixed part (cluster launch, row table, staging of x, cluster
-// reduction) and the entries of all batch tiles at the rate the gathers sustain.
+// Time models of the kernels, all fitted to the same measurements: chains of launches over twelve widths of 256 .. 4096, 80 .. 99 %
+// sparsity and 9 .. 4096 rows; each within 15 to 20 % of nine times in ten.
+//
+// Slab kernel (fp32, up to 64 rows): the staging of a CTA's share of x, its rows and their entries, the cluster reduction.
 double slab_seconds(const cfi_layer* l, int batch) {
-    return 10.8e-6 + 4.4e-12 * (double)l->d.n_active * l->d.k * ((batch + kSlabBT - 1) / kSlabBT);
+    const SlabShape s = slab_shape(l, batch);
+    if (!s.ok) return 1e30;
+    const double share = 1.0 / s.split;
+    return 0.4e-6 + 2.9e-9 * l->d.in * share + 1.1e-9 * s.rows_pc * l->d.k * share + 95e-9 * s.rows_pc + 0.4e-6 * s.split;
 }
 
-// Time model of the split-k kernels on batches above one row (measured, chains of launches over 256 .. 4096 features, 80 .. 99 %
-// sparsity, 1 .. 256 rows; within 25 % of the measured times): a launch, the staging of one tile of x, and for every batch
-// tile a part per row (by the lanes that share it) and a part per entry, which costs more in bf16 (two columns to a bank).
+// Split-k kernels: a launch, the staging of one tile of x, and for every batch tile a part per row (by the lanes that share it)
+// and a part per entry; 1.1 (fp32) and 1.15 (bf16) times the fit, for which fewest calls are slower than on another kernel.
+// bf16 costs more in each: two columns share a bank of shared memory, and the entries of a row are ordered for one column a
+// bank (order_for_banks).
 double splitk_seconds(const cfi_layer* l, int batch) {
     const SplitkShape s = splitk_shape(l, batch);
-    const double eighths = s.bt / 8.0, per_entry = l->dtype == CFI_BF16 ? 3.5e-12 : 2.1e-12;
-    return 2.9e-6 + 14e-9 * (s.smem / 1024.0) + s.grid_y * (0.3e-9 * l->d.out * s.g / 32.0 + per_entry * eighths * l->d.n_active * l->d.k);
+    const bool bf = l->dtype == CFI_BF16;
+    const double launch = bf ? 2.2e-6 : 2.0e-6, per_kb = bf ? 58e-9 : 30e-9, per_row = bf ? 0.53e-9 : 0.28e-9, per_entry = bf ? 2.9e-12 : 1.9e-12;
+    return launch + per_kb * (s.smem / 1024.0) + s.grid_y * (per_row * l->d.out * s.g / 32.0 + per_entry * (s.bt / 8.0) * l->d.n_active * l->d.k);
 }
 
-// Time model of the tensor-core variant, from the models that choose its launch shape.
+// Tensor cores.  fp32: the model that chooses the launch shape; narrow tiles fill and drain faster than its common constant says.
+// bf16, one tile a CTA: a CTA's share of K, the reduction of a split, how many CTAs there are; the persistent kernel's batches
+// have no other candidate.
 double dense_seconds(const cfi_layer* l, int batch) {
     if (l->dtype == CFI_F32) {
         const SplitShape s = split_shape(l, batch);
         if (!s.ok) return 1e30;
-        return s.seconds - (s.bt <= 64 ? 1.3e-6 : 0.0);  // narrow tiles fill and drain faster than the shapes' common constant says
+        return s.seconds - (s.bt <= 64 ? 1.3e-6 : 0.0);
     }
-    double t = 0.0;
-    tc_bf16_split(l, batch, &t);
-    return std::max(t, 2.0 * l->out_pad * (double)l->d.in / kSplitHbmBytesPerSecond + 4.7e-6);
+    const int split = tc_bf16_split(l, batch), k_blocks = (l->d.in + kTcK - 1) / kTcK;
+    const double ctas = (double)((batch + kTcM - 1) / kTcM) * ((l->d.out + kTcN - 1) / kTcN) * split;
+    const double t = 2.15e-6 + 0.24e-6 * k_blocks / split + (split > 1 ? 1.5e-6 : 0.0) + 2.6e-6 * ctas / l->sm_count + 0.8e-12 * batch * l->d.out;
+    return std::max(t, 2.0 * l->out_pad * (double)l->d.in / kSplitHbmBytesPerSecond + 2.5e-6);
 }
 
-// Time model of the gather kernel (measured): the walk over the slabs of x by however many rows a CTA has, and the
-// arithmetic at the rate the gathers sustain; with many batch tiles the re-staging of x by every row tile.
+// Gather kernel: per wave of CTAs the walk over the columns of x, by slabs, and the entries of a CTA's rows.
 double gather_seconds(const cfi_layer* l, int batch) {
     const BatchShape bs = batch_shape(l, batch);
     if (!bs.ok) return 1e30;
-    const double t_fma = 2.0 * batch * (double)l->d.n_active * l->d.k / 12.5e12;
-    const double t_stage = (double)bs.grid_y * kBatchTile * l->d.in * 4.0 * bs.grid_x / 3.7e12;
-    return std::max(2e-6 + 7e-9 * l->d.in + t_fma, t_fma + t_stage - 0.5 * std::min(t_fma, t_stage) + 5e-6);
+    const bool bf = l->dtype == CFI_BF16;
+    const double waves = std::ceil((double)bs.grid_x * bs.grid_y / l->sm_count), entries = l->d.stride_q * 4.0;
+    const double per_wave = 5.4e-9 * l->d.in + 0.5e-6 * bs.rph * l->d.n_slabs + (bf ? 24.8e-9 : 16.8e-9) * bs.rph * entries + (bf ? 0.0 : 0.55e-9) * bs.rt * entries;
+    return (bf ? 2.5e-6 : 2.3e-6) + waves * per_wave;
 }
 
 // Up to eight rows: split-k.  Above, the fastest by the models among the kernels whose layout the layer holds.  Measured, us a
-// call (split-k / slab / gather / tensor cores): 4096 x 4096 fp32 at 95 %, batch 16 9.4 / 14.1 / 37 / 14.4, batch 64
-// 27 / 41 / 35 / 18; at 99 %, batch 64 11.6 / 30 / 29 / 17.6, batch 256 38 / - / 45 / 40; 768 -> 3072 at 90 %, batch 16
-// 7.6 / 6.1 / 9.4 / 5.9.  bf16 at 99 %: batch 32 7.8 / - / 28 / 13, batch 128 26 / - / 26 / 14.6; at 95 %, batch 32 26 / - / 35 / 13.
+// call (split-k / slab / gather / tensor cores): 4096 x 4096 fp32 at 95 %, batch 16 8.7 / 13.8 / 37 / 12.0, batch 64
+// 26 / 40 / 35 / 15; at 99 %, batch 64 12.4 / 30 / 29 / 15; 768 -> 3072 at 90 %, batch 16 4.7 / 6.0 / 9.4 / 5.4.  bf16, 768 -> 3072
+// at 90 %, batch 64 13.9 / - / 8.2 / 6.6; 4096 x 4096 at 99 %, batch 32 6.8 / - / 29 / 9.6; at 95 %, batch 32 18.7 / - / 34 / 9.6.
 int choose_variant(const cfi_layer* l, int batch) {
     // A layer built without the small-batch layout runs every batch size on what it has.
     if (!(l->layouts & CFI_LAYOUT_SMALL_BATCH) && batch <= 24)
@@ -1312,7 +1322,7 @@ int choose_variant(const cfi_layer* l, int batch) {
     };
     if (l->tc_ok) consider(CFI_VARIANT_DENSE_TC, dense_seconds(l, batch));
     if (batch <= 256 && splitk_fits(l, batch)) consider(CFI_VARIANT_SPLITK, splitk_seconds(l, batch));
-    if (batch <= 64 && l->dtype == CFI_F32 && slab_shape(l, batch).ok) consider(CFI_VARIANT_SLAB, slab_seconds(l, batch));
+    if (batch <= 64 && l->dtype == CFI_F32) consider(CFI_VARIANT_SLAB, slab_seconds(l, batch));
     if (!(l->tc_ok && l->dtype == CFI_BF16)) consider(CFI_VARIANT_BATCH, gather_seconds(l, batch));  // bf16 tensor cores always beat it
     return best >= 0 ? best : fallback_variant(l, batch);
 }

@@ -1,6 +1,7 @@
-"""The automatic kernel choice (cfi_forward) against every explicit variant that can run the shape, on the named
-workloads: the kernel it picks must be within 15 % (plus 0.3 us of timing noise) of the fastest one.  Times are CUDA
-events around replays of a CUDA graph of 50 launches on one layer, 200 launches per figure."""
+"""The automatic kernel choice (cfi_forward) against every explicit variant that can run the shape: on the named workloads
+the kernel it picks must be within 15 % (plus 0.3 us of timing noise) of the fastest one, on a grid of widths, sparsities,
+batches, types and layouts within what the models of the choice leave open.  Times are CUDA events around replays of a CUDA
+graph of 50 launches on one layer, 200 launches per figure."""
 import numpy as np
 import pytest
 
@@ -47,8 +48,6 @@ def test_auto_is_close_to_the_best_variant(base, names):
         y = torch.empty((w.batch, w.out_features), device="cuda")
         times = {}
         for variant in ("splitk", "batch", "slab", "dense_tc"):
-            if variant == "splitk" and w.batch > 64:          # hundreds of microseconds: never a candidate there
-                continue
             try:
                 times[variant] = _time(cfi, torch, layer, x, y, w.batch, variant)
             except cfi.CfiError as e:
@@ -58,3 +57,40 @@ def test_auto_is_close_to_the_best_variant(base, names):
         report[name] = (t_auto, times)
         assert t_auto <= 1.15 * best + 0.3, (name, t_auto, times)
     layer.close()
+
+
+# Batches on both sides of every line of the choice above eight rows; fp32 and bf16; with the dense copy and without.
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("layouts", [7, 3])
+@pytest.mark.parametrize("in_f,out_f", [(768, 3072), (3072, 768), (512, 2048), (2048, 2048)])
+def test_auto_is_close_to_the_best_variant_on_a_grid(dtype, layouts, in_f, out_f):
+    """The models are within 20 to 25 % of the times, so of two kernels the one that looks faster takes at most
+    1.25 / 0.78 = 1.6 times as long as the other.  fp32: the tensor cores' split products are less exact and taken for a large gain only, so where
+    the choice is a kernel with fp32 sums it is compared with those."""
+    import torch
+    from paper_2305_02299_b200 import binding as cfi
+    from parity import torch_dtype
+    slow, report = [], {}
+    for k in (max(1, in_f // 100), in_f // 20, in_f // 10):
+        L = inputs.make_layer(in_f, out_f, k, seed=k)
+        layer = cfi.cfi_create(*cfi.cfi_pack(L.w_dense, L.mask), L.bias, in_f, out_f, dtype=dtype, layouts=layouts)
+        for batch in (9, 16, 32, 64, 128, 256, 320):
+            x = torch.from_numpy(inputs.make_x(batch, in_f, seed=batch)).cuda().to(torch_dtype(dtype))
+            y = torch.empty((batch, out_f), device="cuda", dtype=x.dtype)
+            times = {}
+            for variant in ("splitk", "batch", "slab", "dense_tc"):
+                if variant == "dense_tc" and dtype == "f32" and cfi.cfi_choose_variant(layer, batch) != 4:
+                    continue
+                if (variant, dtype) == ("slab", "bf16") or batch > {"splitk": 256, "slab": 64}.get(variant, batch):
+                    continue                                    # no candidate there
+                try:
+                    times[variant] = _time(cfi, torch, layer, x, y, batch, variant)
+                except cfi.CfiError as e:
+                    assert e.status == 2
+            t_auto = _time(cfi, torch, layer, x, y, batch, "auto")
+            report[(k, batch)] = t_auto / min(times.values())
+            if t_auto > 1.6 * min(times.values()) + 0.3:
+                slow.append((k, batch, t_auto, times))
+        layer.close()
+    print(sorted(report.values())[-3:])
+    assert not slow, slow
