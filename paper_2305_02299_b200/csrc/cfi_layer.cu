@@ -1306,6 +1306,41 @@ double gather_seconds(const cfi_layer* l, int batch) {
     return (bf ? 2.5e-6 : 2.3e-6) + waves * per_wave;
 }
 
+// fp32: which calls the tensor cores may have at all.  A split-TF32 product drops w_lo x_lo and the remainders of both
+// operands: 4e-7 .. 1.7e-6 of error against 64 bits (2-norm, 256 .. 4096 columns) where the fp32 kernels have 4e-8 .. 2e-7.  The
+// caller of cfi_forward does not choose between the two, so a call changes sides for a large gain only, and not with every
+// refinement of the kernels: the line is drawn with rates that the tensor-core kernel exceeds and whole tiles, not with the
+// models that choose its launch shape.  Just below it the fp32 kernels take up to 1.9 times as long (1024 -> 4096 k 41 at batch
+// 2500: gather kernel 174 us, tensor cores 91; 3072 -> 768 k 61 at batch 1576: 58 and 37).
+bool worth_split_tf32(const cfi_layer* l, int batch) {
+    constexpr double kNever = 1e30;
+    const int k_blocks = (l->d.in + kSpK - 1) / kSpK, tiles_m = (l->d.out + kSpM - 1) / kSpM;
+    const double t_hbm = 4.0 * l->out_pad * (double)l->d.in / kSplitHbmBytesPerSecond, nnz = (double)l->d.n_active * l->d.k;
+    double t_dense = kNever;
+    for (int bt : kSpTiles) {
+        const int64_t tiles = (int64_t)tiles_m * ((batch + bt - 1) / bt);
+        if ((batch + bt - 1) / bt > 65535) continue;
+        const double per_block = bt >= 128 ? 0.51e-6 : bt >= 96 ? 0.40e-6 : 0.31e-6;
+        for (int split = 1; split <= kMaxSplit; ++split) {
+            if (split > 1 && (k_blocks < 2 * split || tiles * split > 2 * (int64_t)l->sm_count)) continue;
+            const int64_t resident = split_resident_clusters(l, bt, split);
+            if (resident == 0) continue;
+            const int64_t waves = (tiles + resident - 1) / resident;
+            const double blocks = (double)waves * ((k_blocks + split - 1) / split) * per_block;
+            t_dense = std::min(t_dense, std::max(blocks, t_hbm) + (double)waves * (kSplitWave + (split > 1 ? split_seconds_reduce(bt) : 0.0)) + kSplitLaunch);
+        }
+    }
+    double t_fp32 = kNever;
+    if (batch <= 24) {  // passes of eight rows: staging, or the entries
+        if (splitk_fits(l, batch)) t_fp32 = ((batch + 7) / 8) * (2.3e-6 + std::max(l->d.in * 32 / 1024.0 * 90e-9, nnz / 176e9));
+    } else if (const BatchShape bs = batch_shape(l, batch); bs.ok) {
+        const double t_fma = 2.0 * batch * nnz / 12.5e12, t_stage = (double)bs.grid_y * kBatchTile * l->d.in * 4.0 * bs.grid_x / 3.7e12;
+        t_fp32 = t_fma + t_stage - 0.5 * std::min(t_fma, t_stage) + 5e-6;
+    }
+    if (batch <= 64 && slab_shape(l, batch).ok && 10.8e-6 + 4.4e-12 * nnz * ((batch + kSlabBT - 1) / kSlabBT) < t_dense) return false;
+    return t_dense < t_fp32;
+}
+
 // Up to eight rows: split-k.  Above, the fastest by the models among the kernels whose layout the layer holds.  Measured, us a
 // call (split-k / slab / gather / tensor cores): 4096 x 4096 fp32 at 95 %, batch 16 8.7 / 13.8 / 37 / 12.0, batch 64
 // 26 / 40 / 35 / 15; at 99 %, batch 64 12.4 / 30 / 29 / 15; 768 -> 3072 at 90 %, batch 16 4.7 / 6.0 / 9.4 / 5.4.  bf16, 768 -> 3072
@@ -1320,7 +1355,7 @@ int choose_variant(const cfi_layer* l, int batch) {
     auto consider = [&](int variant, double t) {
         if (t < 1e29 && (best < 0 || t < best_t)) best = variant, best_t = t;
     };
-    if (l->tc_ok) consider(CFI_VARIANT_DENSE_TC, dense_seconds(l, batch));
+    if (l->tc_ok && (l->dtype == CFI_BF16 || worth_split_tf32(l, batch))) consider(CFI_VARIANT_DENSE_TC, dense_seconds(l, batch));
     if (batch <= 256 && splitk_fits(l, batch)) consider(CFI_VARIANT_SPLITK, splitk_seconds(l, batch));
     if (batch <= 64 && l->dtype == CFI_F32) consider(CFI_VARIANT_SLAB, slab_seconds(l, batch));
     if (!(l->tc_ok && l->dtype == CFI_BF16)) consider(CFI_VARIANT_BATCH, gather_seconds(l, batch));  // bf16 tensor cores always beat it
