@@ -512,7 +512,8 @@ def dense_shape(cfi, layer, batch):
 
 def kernel_name(variant, shape=None, dtype="f32"):
     if variant == "dense_tc":
-        return f"cfi_dense_split_kernel<{shape['batch_tile']}>" if shape else "cfi_dense_split_kernel"
+        # tiles of 80 and 112 rows run on the kernel's tiles of 96 and 128
+        return f"cfi_dense_split_kernel<{ {80: 96, 112: 128}.get(shape['batch_tile'], shape['batch_tile'])}>" if shape else "cfi_dense_split_kernel"
     return {"batch": "cfi_batch_kernel<float>", "splitk": "cfi_splitk_kernel<float>", "simple": "cfi_simple_kernel<float>",
             "slab": "cfi_slab_kernel<float>"}[variant]
 

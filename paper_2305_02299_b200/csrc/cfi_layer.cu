@@ -1002,13 +1002,13 @@ struct SplitShape {
 
 // Batch tile and K split: a narrower batch tile costs less per K block, a wider one shares each weight box among more
 // batch rows; splitting K over a cluster fills the SMs that the tiles alone would leave idle, as long as every CTA
-// still gets a few K blocks.  force_bt / force_split (0 = free) pin one or both.
-SplitShape split_shape(const cfi_layer* l, int batch, int force_bt = 0, int force_split = 0) {
+// still gets a few K blocks.  force_rows / force_split (0 = free) pin one or both.
+SplitShape split_shape(const cfi_layer* l, int batch, int force_rows = 0, int force_split = 0) {
     const int k_blocks = (l->d.in + kSpK - 1) / kSpK, tiles_m = (l->d.out + kSpM - 1) / kSpM;
     const double t_hbm = 4.0 * l->out_pad * (double)l->d.in / kSplitHbmBytesPerSecond;
     SplitShape best{128, 128, 1, 0.0, false};
     for (int rows = kSpRowStep; rows <= 128; rows += kSpRowStep) {
-        if (force_bt && rows != force_bt) continue;
+        if (force_rows && rows != force_rows) continue;
         const int bt = *std::lower_bound(std::begin(kSpTiles), std::end(kSpTiles), rows);
         const int64_t tiles_b = (batch + rows - 1) / rows;
         if (tiles_b > 65535) continue;
@@ -1038,11 +1038,11 @@ cfi_status_t launch_dense_split_bt(const cfi_layer* l, const SplitShape& sh, con
                               l->map_w, map_x, static_cast<float*>(y), batch, sh.rows);
 }
 
-cfi_status_t launch_dense_split(const cfi_layer* l, const void* x, void* y, int batch, cudaStream_t st, int force_bt = 0,
+cfi_status_t launch_dense_split(const cfi_layer* l, const void* x, void* y, int batch, cudaStream_t st, int force_rows = 0,
                                 int force_split = 0) {
-    if (force_bt && split_bt_index(force_bt) < 0) return CFI_ERR_SHAPE;
+    if (force_rows && (force_rows < kSpRowStep || force_rows > 128 || force_rows % kSpRowStep)) return CFI_ERR_SHAPE;
     if (force_split < 0 || force_split > kMaxSplit) return CFI_ERR_SHAPE;
-    const SplitShape sh = split_shape(l, batch, force_bt, force_split);
+    const SplitShape sh = split_shape(l, batch, force_rows, force_split);
     if (!sh.ok) return CFI_ERR_SHAPE;
     switch (sh.bt) {
         case 16: return launch_dense_split_bt<16>(l, sh, x, y, batch, st);
@@ -1109,7 +1109,7 @@ int tc_bf16_split(const cfi_layer* l, int batch, double* seconds = nullptr) {
     return best;
 }
 
-// tile / cluster: 0 = chosen here.  fp32 layers: tile = batch rows per tile (16, 32, 64, 128); bf16 layers: tile = outputs
+// tile / cluster: 0 = chosen here.  fp32 layers: tile = batch rows per tile (16, 32, .. 128); bf16 layers: tile = outputs
 // per tile, 128 (one tile per CTA, K may be split over `cluster` CTAs) or 256 (persistent kernel, no split).
 cfi_status_t launch_dense_tc(const cfi_layer* l, const void* x, void* y, int batch, cudaStream_t st, int tile = 0,
                              int cluster = 0) {
@@ -1776,7 +1776,7 @@ extern "C" cfi_status_t cfi_dense_tile_shape(const cfi_layer_t* layer, int32_t b
     } else {
         const SplitShape sh = split_shape(layer, batch);
         if (!sh.ok) return CFI_ERR_SHAPE;
-        *tile_n = sh.bt, *cluster = sh.split;
+        *tile_n = sh.rows, *cluster = sh.split;
     }
     return CFI_OK;
 }

@@ -31,14 +31,14 @@ def test_dense_tc_matches_oracle(in_f, out_f, k, nabl, B, act, dtype):
     assert_parity(y, y_ref, S, dtype)
 
 
-# fp32: every batch tile (16, 32, 48, 64, 96, 128 rows; the MMAs are 2 x and 1 x that wide) with and without a K split over a
+# fp32: every batch tile (16, 32, .. 128 rows, 80 and 112 of them tiles used in part) with and without a K split over a
 # thread-block cluster, on shapes with ragged output, batch and K tails, few and many K blocks per CTA (more blocks
 # than ring stages, fewer blocks than CTAs of the cluster), ablated rows and both activations.
 SPLIT_SHAPES = [(768, 384, 77, 19, 200, "gelu"), (3072, 200, 307, 20, 70, "none"), (1000, 72, 100, 5, 257, "gelu"),
                 (520, 640, 52, 30, 129, "none"), (64, 8, 5, 1, 5, "gelu"), (40, 136, 1, 7, 33, "none")]
 
 
-@pytest.mark.parametrize("tile", [16, 32, 48, 64, 96, 128])
+@pytest.mark.parametrize("tile", [16, 32, 48, 64, 80, 96, 112, 128])
 @pytest.mark.parametrize("cluster", [1, 2, 3, 4, 8])
 def test_dense_split_tf32_every_launch_shape(tile, cluster):
     from paper_2305_02299_b200 import binding as cfi
@@ -65,14 +65,16 @@ def test_dense_split_tf32_tiles_used_in_part(in_f, out_f, k, nabl, B, act):
     x = inputs.make_x(B, in_f, seed=B)
     y_ref, S = oracle_layer(L, x, "f32", act)
     dl = device_layer(L, "f32", act)
-    assert cfi.cfi_dense_tile_shape(dl, B)[0] in (96, 128)
+    shape = cfi.cfi_dense_tile_shape(dl, B)
+    assert shape[0] in (80, 112), shape
     y = run_device(dl, x, "f32", "dense_tc")
+    assert np.array_equal(y, run_device(dl, x, "f32", dense_shape=shape))     # the shape that is reported is the one that runs
     assert cfi.cfi_device_status(dl) == 0
     dl.close()
     assert scaled_error(y, y_ref, S) <= TOL["f32"]
 
 
-@pytest.mark.parametrize("tile,cluster", [(16, 4), (48, 4), (64, 8), (96, 2), (128, 2), (32, 1)])
+@pytest.mark.parametrize("tile,cluster", [(16, 4), (48, 4), (64, 8), (96, 2), (128, 2), (32, 1), (80, 1), (80, 3), (112, 2)])
 def test_dense_split_tf32_chain_of_launches(tile, cluster):
     """Back-to-back launches (a CUDA graph of 48 calls over 6 rotating layers; each launch lets its successor start
     early and waits for its predecessor before it reads x): a long K, so that the ring wraps several times per CTA.
