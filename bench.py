@@ -436,9 +436,9 @@ def main():
                          "frac": achieved_tflops / ceil_.fma_tflops,
                          # dram__bytes_read.sum + dram__bytes_write.sum of one launch, from the ncu capture summarised
                          # under profiles/ for exactly this kernel and launch shape; null otherwise
-                         "traffic": CAPTURED_TRAFFIC.get((w.name, kernel_name(chosen, shape), json.dumps(shape))),
+                         "traffic": CAPTURED_TRAFFIC.get((w.name, kernel_name(chosen, shape, w.batch), json.dumps(shape))),
                          "peak_source": ceil_.fma_source,
-                         "kernel": kernel_name(chosen, shape),
+                         "kernel": kernel_name(chosen, shape, w.batch),
                          "note": "bound/peak are the sparse problem's own roofline (2*B*n_active*k FMAs on the fp32 FMA "
                                  "pipes, the bound of the gather formulation; its shared-memory ceiling is given beside "
                                  "it); when the chosen kernel is the tensor-core variant the dense flops it executes are "
@@ -492,9 +492,22 @@ def main():
         line["stack_batch1"] = stack_batch1_leg(cfi, torch, l2, peaks)
         line["srigl_update"] = srigl_update_leg(cfi, torch, peaks)
     if rank == 0:
-        print(json.dumps(line))
+        headline, legs = split_line(line)
+        for name, leg in legs.items():
+            print(json.dumps({name: leg}), file=sys.stderr)
+        print(json.dumps(headline))
     if dist:
         dist.destroy_process_group()
+
+
+# The legs that a default run adds to its headline.  Together they are some 20 KB of JSON, too long a line for a reader that
+# keeps only the end of the output, so each goes to stderr as a line of its own and stdout has the one line of the contract.
+LEGS = ("floor", "sweep", "batch1", "context", "stack_c5", "batch2048", "device_probe", "stack_batch1", "srigl_update")
+
+
+def split_line(line):
+    """(what is printed as the one line on stdout, the legs)"""
+    return {k: v for k, v in line.items() if k not in LEGS}, {k: line[k] for k in LEGS if k in line}
 
 
 VARIANT_NAMES = {1: "simple", 2: "splitk", 3: "batch", 4: "dense_tc", 5: "slab"}
@@ -510,11 +523,12 @@ def dense_shape(cfi, layer, batch):
     return {"batch_tile": tile, "cluster_k_split": cluster}
 
 
-def kernel_name(variant, shape=None, dtype="f32"):
+def kernel_name(variant, shape=None, batch=1):
+    """The kernel that runs an fp32 layer with this variant."""
     if variant == "dense_tc":
         # tiles of 80 and 112 rows run on the kernel's tiles of 96 and 128
         return f"cfi_dense_split_kernel<{ {80: 96, 112: 128}.get(shape['batch_tile'], shape['batch_tile'])}>" if shape else "cfi_dense_split_kernel"
-    return {"batch": "cfi_batch_kernel<float>", "splitk": "cfi_splitk_kernel<float>", "simple": "cfi_simple_kernel<float>",
+    return {"batch": "cfi_batch_kernel<float>", "splitk": "cfi_splitk_kernel" if batch == 1 else "cfi_splitk_rows_kernel<float>", "simple": "cfi_simple_kernel<float>",
             "slab": "cfi_slab_kernel<float>"}[variant]
 
 

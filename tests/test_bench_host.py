@@ -51,6 +51,16 @@ def test_byte_and_flop_models_match_the_stated_figures():
     assert abs(bench.algorithmic_bytes(w["c2"], 3072) / 1e6 - 5.849) < 0.001
 
 
+def test_default_run_prints_the_contract_line_alone():
+    """The legs of a default run leave the line on stdout; what the line must have stays."""
+    keys = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling", "vs_baseline", "dtype", "data",
+            "config", "roofline", "e2e", "gpu_launches", "clocks", "cpu_baseline", "variants_us")
+    line = {**{k: 1 for k in keys}, **{k: {"x": list(range(500))} for k in bench.LEGS}}
+    headline, legs = bench.split_line(line)
+    assert tuple(headline) == keys and set(legs) == set(bench.LEGS) and all(legs[k] == line[k] for k in legs)
+    assert bench.split_line({"value": 1}) == ({"value": 1}, {})
+
+
 def test_reference_arm_prints_one_json_line():
     r = subprocess.run([sys.executable, os.path.join(ROOT, "bench.py"), "--impl", "reference", "--steps", "2", "--warmup", "1"],
                        capture_output=True, text=True, timeout=300)
