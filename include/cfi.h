@@ -348,8 +348,8 @@ cfi_status_t cfi_destroy(cfi_layer_t* layer);
  *
  * A bf16 chain with widths that are no multiple of 8 (layers in the compact output form, say), made of layers that were
  * created with CFI_LAYOUT_DENSE, keeps dense copies with those widths rounded up beside its buffers (2 * in * out bytes for
- * each such layer): batches above 24 rows then run on the tensor cores like any other bf16 layer, with CFI_VARIANT_DENSE_TC's
- * treatment of non-finite inputs.
+ * each such layer): batches above 24 rows then run on the tensor cores at every sparsity, with CFI_VARIANT_DENSE_TC's treatment of
+ * non-finite inputs (layers of such widths called one by one, or created without CFI_LAYOUT_DENSE, run on the condensed kernels).
  *
  * cfi_stack_forward enqueues the n_layers forwards on `stream` without synchronising; batch above
  * max_batch returns CFI_ERR_BUFFER_TOO_SMALL.  One stack must not run on two streams at once (the

@@ -1898,9 +1898,12 @@ namespace {
 // activations between the layers are the stack's own, so their rows may be as long as that needs: a bf16 layer with an odd
 // width (the compact output form leaves any number of neurons) gets a twin with both widths rounded up, on zero weights and
 // zero biases, and the chain runs on the dense copies of these.  An odd input or output of the whole chain is copied from
-// or to rows of its own length.  Only for batches that the tensor cores take for any even-width bf16 layer too (above 24
-// rows); fp32 chains stay on the gather kernels, whose sums the split-TF32 products do not match over a long fan-in.
-// 768 -> 2918 (GELU) -> 768 at batch 197: 83 us on the gather kernels, 18 us on twins.
+// or to rows of its own length.  From 25 rows on, whatever the sparsity, so that every such batch of a chain runs on one kind
+// of kernel; very sparse chains of up to about a hundred rows would be faster on split-k.  Measured, us a chain on twins / layer
+// by layer without them: 768 -> 2918 (GELU) -> 768 at batch 197 18 / 83 (k 77 and 307); 768 -> 2918 -> 768 at 90 %, batch 32
+// 11.9 / 18.2, batch 256 17.2 / 82; at 99 %, batch 32 11.9 / 13.1, batch 64 13.2 / 11.1; 1000 -> 1501 -> 1000 at 99 %, batch 32
+// 11.5 / 8.1, batch 256 16.8 / 13.8; 513 -> 2001 -> 513, whose ends are copied, at 90 %, batch 32 14.1 / 12.2, batch 256 21.7 / 74.
+// fp32 chains stay on the fp32 kernels, whose sums the split-TF32 products do not match over a long fan-in.
 constexpr int kTwinBatch = 25;
 int round8(int width) { return (width + 7) & ~7; }
 

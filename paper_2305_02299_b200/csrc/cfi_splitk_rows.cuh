@@ -5,11 +5,14 @@
 // memory.  With 100 KB of x (8 rows of 3072 columns), transposed to [column][BT] on the way, that was six dependent round
 // trips to L2 per CTA, most of the call.  Here x stays as it is, xs[b][column] in its own type: 16-byte asynchronous copies
 // put all of it in flight at once and cost neither registers nor conversions.  A gathered entry takes BT loads of 4 (or 2)
-// bytes instead of one or two of 16; the same number of shared-memory wavefronts, since the order of a row's entries keeps
-// the lanes of an instruction in different banks for one row of x (order_for_banks), which no wider gather can profit from.
+// bytes instead of one or two of 16, which is the same number of shared-memory wavefronts where the lanes of an instruction
+// meet different banks.  They do so in part only: order_for_banks deals a row's entries by column mod 32 to the lanes that
+// share the row at batch 1, and here more lanes share it as the tile grows, and in bf16 two columns share a bank.
+// Wavefronts an instruction, from the placement: fp32 3072 columns k 307 1.5, 4096 k 205 1.8 (tiles of 4 and 8) and 2.0, 768
+// k 77 2.3 .. 2.5 and 3.6; bf16 2.5 and 3.2, 3.4 and 4.2, 3.0 .. 3.3 and 4.5.
 //
-// 3072 -> 768, k 307, per call in a chain of launches: batch 8 fp32 10.2 -> 5.0 us, bf16 18.4 -> 6.2;
-// batch 2 fp32 5.0 -> 2.8; batch 1 bf16 6.7 -> 1.8.  4096 x 4096 at 80 %, batch 8: 16.5 -> 12.2 us.
+// 3072 -> 768, k 307, per call in a chain of launches, against x transposed to [column][BT] by the threads: batch 8 fp32
+// 10.2 -> 3.7 us, bf16 18.2 -> 4.1; batch 2 fp32 4.7 -> 2.5; batch 1 bf16 6.6 -> 1.7.  4096 x 4096 at 80 %, batch 8: 15.7 -> 11.9 us.
 
 __device__ __forceinline__ void cp_async4(uint32_t smem_off, const void* gmem_src) {
     const uint32_t d = (uint32_t)__cvta_generic_to_shared(smem_at(smem_off));
@@ -24,7 +27,8 @@ __host__ __device__ inline int splitk_rows_pitch(int in, int elem) {
 }
 
 // Units a lane takes at a time: a unit costs BT times the instructions of batch 1, so more lanes share a row instead, each
-// with less to do (768 -> 3072 at batch 8 with 4 units a lane: six warps per SM, 840 instructions each, 5.6 us; with one 4.7).
+// with less to do (768 -> 3072 at batch 8 in one tile of 8, 4 units a lane: six warps per SM, 840 instructions each, 5.6 us; with
+// one 4.7; in two tiles of 4 with two units 3.3).
 __host__ __device__ constexpr int splitk_rows_units(bool fp32_values, bool idx16, int bt) {
     const int u = splitk_units_in_flight(fp32_values, idx16);
     return bt <= 2 ? u : bt == 4 ? u / 2 : 1;
