@@ -48,6 +48,16 @@ def test_small_batch_rows_of_x(in_f, out_f, k, dtype):
         check_layer(L, inputs.make_x(B, in_f, seed=B), dtype, variants=("splitk",))
 
 
+@pytest.mark.parametrize("in_f,out_f,k", [(8, 40, 3), (2918, 64, 280), (3333, 24, 2000), (4100, 33, 1), (3072, 520, 3000)])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_small_batch_tiles_at_their_borders(in_f, out_f, k, dtype):
+    """The same on both sides of batch 128, where tiles of 4 rows give way to tiles of 8, full and in part; 3072 x 520 with 1.56 M
+    entries has 16-bit columns."""
+    L = inputs.make_layer(in_f, out_f, k, n_ablated=out_f // 9 if k < 3000 else 0, seed=in_f)
+    for B in (127, 128, 129, 136):
+        check_layer(L, inputs.make_x(B, in_f, seed=B), dtype, variants=("splitk",))
+
+
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("act", ["none", "gelu"])
 def test_gelu_and_ablated_rows(dtype, act):
