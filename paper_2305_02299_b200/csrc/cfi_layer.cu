@@ -698,7 +698,7 @@ SplitkShape splitk_shape(const cfi_layer* l, int batch) {
         // As few CTAs per SM as give every lane a row (at most 512 lanes each, what fits beside the staged x), the rows
         // spread evenly over them: 5.2 rows of 768 on each of 148 SMs rather than 16 rows on 48.  No more than the registers
         // let an SM hold (two of 64 a thread; tiles of 1 and 2 rows take up to 82): a CTA that has to wait for another to end
-        // stages x all over (768 -> 3072 at batch 16: 7.5 us with three, 4.5 with two).
+        // stages x all over (768 -> 3072 at batch 16: 5.9 us with three, 4.5 with two).
         const int64_t lanes_per_sm = (lanes * s.grid_y + l->sm_count - 1) / l->sm_count;
         const int per_sm = (int)std::max<int64_t>(1, std::min<int64_t>({fit, s.bt >= 4 ? 2 : 1, (lanes_per_sm + 511) / 512}));
         const int slots = std::max(1, l->sm_count * per_sm / s.grid_y);
